@@ -250,6 +250,7 @@ MlpDims make_dims(int K, int H0, int H1, int NA, bool sparse) {
   m.ob3 = o; o += m.NOP;
   m.sparse = sparse ? 1 : 0;
   m.oC = o; o += sparse ? H0 : 0;
+  m.oFin = o; o += 1;
   m.stride = align_up(o, 4);
   return m;
 }
@@ -298,6 +299,13 @@ aht_status pack_policy(const MlpDims& m, const void* const* W, const void* const
     if (!host_view(b[l], (size_t)outs[l] * esz, &src)) return fail(AHT_ECUDA, "copying biases failed");
     for (int n = 0; n < outs[l]; ++n) dst[ob[l] + n] = to_f32(src, n, dtype);
   }
+  uint32_t odd = 0;  // an exponent of all ones (infinity, NaN) anywhere in W1
+  for (int64_t i = 0; i < (int64_t)m.K * m.H0; ++i) {
+    uint32_t u;
+    std::memcpy(&u, &dst[m.oW1 + i], 4);
+    odd |= (u & 0x7F800000u) == 0x7F800000u ? 1u : 0u;
+  }
+  dst[m.oFin] = odd ? 0.0f : 1.0f;
   if (m.sparse) {  // c = b1 + W1 x_default in fp64, rounded once
     for (int n = 0; n < m.H0; ++n) {
       double acc = dst[m.ob1 + n];
@@ -660,21 +668,33 @@ aht_status xplay_lbf_tc(aht_ctx* c, const int32_t* ego_ids, int32_t n_ego, const
   return AHT_OK;
 }
 
-// Tile rows for an M-row launch that fits in shared memory (M multiple of 4).
+// Shared memory of a tile of the CUDA-core rollout kernels.
+size_t tile_smem(const aht_ctx* c, const TileCfg& t) {
+  const bool turn = c->env.kind == AHT_HANABI || c->env.kind == AHT_MINI_HANABI;
+  return (size_t)smem_layout(t, c->mlp, c->ops.bytes(), turn ? 1 : 2, 2, c->env.kind != AHT_LBF).total;
+}
+
+// The tile of M rows, with the output layers on chip where shared memory has room for them.
+TileCfg tile_cfg(const aht_ctx* c, int M) {
+  const TileCfg t{M, 1};
+  return tile_smem(c, t) <= c->smem_optin ? t : TileCfg{M, 0};
+}
+
+// Rows of a tile for up to `want` rows that fits in shared memory (8, 16 or 24).
 int fit_rows(const aht_ctx* c, int want) {
-  int M = (int)align_up(want, 4);
-  while (M > 4 && (size_t)smem_layout(M, c->mlp, c->ops.bytes()).total > c->smem_optin) M = (int)align_up(M / 2, 4);
+  int M = std::min((int)align_up(want, 8), kMaxTileRows);
+  while (M > 8 && tile_smem(c, TileCfg{M, 0}) > c->smem_optin) M -= 8;
   return M;
 }
 
-// The CUDA-core kernels are latency-bound per CTA: halve the tile (down to 32 rows)
-// while every tile of the launch still fits in one wave of resident CTAs, so that more
-// SMs, and more CTAs per SM, share the work.  tiles(M): the launch's tile count.
+// The CUDA-core kernels are latency-bound per CTA: cut the tile (down to 8 rows) while
+// every tile of the launch still fits in one wave of resident CTAs, so that more SMs, and
+// more CTAs per SM, share the work.  tiles(M): the launch's tile count.
 template <class F>
 int spread_rows(const aht_ctx* c, int M, int which, F tiles) {
-  while (M >= 64) {
-    const int M2 = (int)align_up(M / 2, 4);
-    const int per_sm = c->ops.occupancy(which, smem_layout(M2, c->mlp, c->ops.bytes()).total);
+  while (M > 8) {
+    const int M2 = M - 8;
+    const int per_sm = c->ops.occupancy(which, tile_smem(c, tile_cfg(c, M2)));
     if (per_sm < 1 || tiles(M2) > (int64_t)per_sm * c->n_sms) break;
     M = M2;
   }
@@ -1018,7 +1038,7 @@ static aht_status rollout_common(aht_ctx* c, int32_t ego_id, const int32_t* pool
   a.n_envs = c->n_envs;
   a.perm = c->perm;
   a.tiles = c->tiles;
-  a.M = M;
+  a.cfg = tile_cfg(c, M);
   a.ego = ego_id;
   a.step0 = (uint32_t)c->step;
   a.T = T;
@@ -1065,7 +1085,7 @@ static aht_status rollout_common(aht_ctx* c, int32_t ego_id, const int32_t* pool
     AHT_CUDA(lbf_ppo_tc(ta, grid, tc_smem, c->stream));
     timer_end(c, tk);
   } else {
-    const size_t smem = smem_layout(M, c->mlp, c->ops.bytes()).total;
+    const size_t smem = tile_smem(c, a.cfg);
     const int tk = timer_begin(c);
     AHT_CUDA(c->ops.ppo(a, grid, smem, c->stream));
     timer_end(c, tk);
@@ -1106,8 +1126,8 @@ aht_status aht_rollout_resample(aht_ctx* c, int32_t ego_id, const int32_t* pool,
   // the gathered per-episode tiles run on the dense-first-layer tensor-core kernel; the
   // sparse-first-layer contexts (LBF beyond 256 tensor-memory columns) on CUDA cores
   const bool use_tc = c->tc && !c->tcd.sparse;
-  const int M = use_tc ? 128 : fit_rows(c, 128);
   const int64_t N = c->n_envs;
+  const int M = use_tc ? 128 : spread_rows(c, fit_rows(c, 128), 0, [&](int m) -> int64_t { return resample_tiles(N, m, pool_size); });
   const int od = c->env.obs_dim;
   const int grid = resample_tiles(N, M, pool_size);
   float* last_value = out->last_value ? out->last_value : (out->advantages ? c->last_value : nullptr);
@@ -1201,13 +1221,13 @@ aht_status aht_rollout_resample(aht_ctx* c, int32_t ego_id, const int32_t* pool,
       a.n_envs = N;
       a.perm = c->perm;
       a.tiles = c->tiles;
-      a.M = M;
+      a.cfg = tile_cfg(c, M);
       a.ego = ego_id;
       a.step0 = step;
       a.T = 1;
       a.ep_step = c->ep_step;
       a.traj = tp;
-      const size_t smem = smem_layout(M, c->mlp, c->ops.bytes()).total;
+      const size_t smem = tile_smem(c, a.cfg);
       const int tk = timer_begin(c);
       AHT_CUDA(c->ops.ppo(a, grid, smem, c->stream));
       timer_end(c, tk);
@@ -1273,13 +1293,13 @@ aht_status aht_xplay_matrix(aht_ctx* c, const int32_t* ego_ids, int32_t n_ego,
   a.max_steps = max_steps;
   for (int i = 0; i < n_ego; ++i) a.ego_ids[i] = ego_ids[i];
   for (int j = 0; j < n_tm; ++j) a.tm_ids[j] = tm_ids[j];
-  a.M = M;
+  a.cfg = tile_cfg(c, M);
   a.tiles_per_pair = (envs_per_pair + M - 1) / M;
   a.step0 = (uint32_t)c->step;
   a.returns = out->returns ? out->returns : c->xp_returns;
   a.steps = out->steps;
   a.actions = out->actions;
-  const size_t smem = smem_layout(M, c->mlp, c->ops.bytes()).total;
+  const size_t smem = tile_smem(c, a.cfg);
   const int64_t grid = n_pairs * a.tiles_per_pair;
   if (grid > INT32_MAX) return fail(AHT_EINVAL, "too many tiles");
   const int tk = timer_begin(c);
@@ -1365,13 +1385,13 @@ aht_status aht_xplay_matrix_static(aht_ctx* c, const int32_t* ego_ids, int32_t n
   a.max_steps = max_steps;
   for (int i = 0; i < n_ego; ++i) a.ego_ids[i] = ego_ids[i];
   for (int j = 0; j < n_tm; ++j) a.tm_ids[j] = tm_ids[j];
-  a.M = M;
+  a.cfg = tile_cfg(c, M);
   a.tiles_per_pair = (envs_per_pair + M - 1) / M;
   a.step0 = (uint32_t)c->step;
   a.returns = scratch;  // every entry the reduction reads is written first by this call
   a.steps = nullptr;
   a.actions = nullptr;
-  const size_t smem = smem_layout(M, c->mlp, c->ops.bytes()).total;
+  const size_t smem = tile_smem(c, a.cfg);
   const int64_t grid = n_pairs * a.tiles_per_pair;
   if (grid > INT32_MAX) return fail(AHT_EINVAL, "too many tiles");
   AHT_CUDA(c->ops.xplay(a, (int)grid, smem, c->stream));
@@ -1451,12 +1471,25 @@ aht_status aht_policy_forward(aht_ctx* c, int32_t policy, const uint8_t* obs, in
   if (policy < 0 || policy >= c->n_policies) return fail(AHT_EINVAL, "policy out of range");
   if (n < 1) return fail(AHT_EINVAL, "n must be >= 1");
   DeviceGuard g(c->device);
-  PolicyArgs a{batch_of(c), policy, obs, n, out, 0};
-  a.M = fit_rows(c, 64);
-  const size_t smem = smem_layout(a.M, c->mlp, 0).total;
-  const int64_t grid = (n + a.M - 1) / a.M;
+  PolicyArgs a{batch_of(c), policy, obs, n, out, {}};
+  // Rows per CTA: the launch takes about waves x rows (the FMA pipe of an SM works through
+  // its tiles' rows), so the row count that minimises it; ties to the larger tile, which
+  // reads the weights less often.
+  auto smem_of = [&](const TileCfg& t) { return (size_t)smem_layout(t, c->mlp, 0, 1, 0, false).total; };
+  int64_t best = -1;
+  for (int M = 8; M <= kMaxTileRows; M += 8) {
+    const TileCfg t{M, 0};
+    if (smem_of(t) > c->smem_optin) break;
+    const int64_t tiles = (n + M - 1) / M, cost = (tiles + c->n_sms - 1) / c->n_sms * M;
+    if (best < 0 || cost <= best) {
+      best = cost;
+      a.cfg = t;
+    }
+    if (tiles <= 1) break;
+  }
+  const int64_t grid = (n + a.cfg.M - 1) / a.cfg.M;
   if (grid > INT32_MAX) return fail(AHT_EINVAL, "n too large");
-  AHT_CUDA(launch_policy(a, (int)grid, smem, c->stream));
+  AHT_CUDA(launch_policy(a, (int)grid, smem_of(a.cfg), c->stream));
   return AHT_OK;
 }
 

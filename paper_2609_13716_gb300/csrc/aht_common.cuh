@@ -8,7 +8,6 @@
 
 namespace aht {
 
-constexpr int kThreads = 256;       // threads per CTA of the rollout kernels
 constexpr int kMaxPool = 256;       // teammate pool entries passed by value
 constexpr int kMaxXpIds = 64;       // ego / teammate ids per cross-play call
 
@@ -42,7 +41,15 @@ struct MlpDims {
   // features, c = b1 + W1 x_default kept per policy at oC.
   int32_t sparse;
   int64_t oC;
+  // 1.0 when every weight of W1 is finite (a zero feature then adds nothing to a sum), else 0
+  int64_t oFin;
 };
+// Tiles of the CUDA-core kernels: M rows (8, 16 or 24); w3: the policies' output layers kept
+// in shared memory.
+struct TileCfg {
+  int32_t M, w3;
+};
+constexpr int kMaxTileRows = 24;
 constexpr uint32_t kSparseDefaultWord = 0x01000000u;
 constexpr int kSparseCap = 32;  // list entries per row: a count and up to 31 changed features
 

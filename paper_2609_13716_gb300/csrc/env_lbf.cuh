@@ -13,6 +13,7 @@ namespace aht {
 struct EnvLbf {
   static constexpr bool kTurnBased = false;
   static constexpr int kNumActions = 6;
+  static constexpr bool kBinaryObs = false;  // level-scaled bytes
   struct State {
     uint8_t ax[2], ay[2];
     uint8_t al[2], F, eaten;  // eaten: bit k set when food k is gone (absent foods too)

@@ -13,6 +13,7 @@ namespace aht {
 struct EnvMiniHanabi {
   static constexpr bool kTurnBased = true;
   static constexpr int kNumActions = 10;
+  static constexpr bool kBinaryObs = true;  // observations are bit rows on chip
   static constexpr int kTurnCap = 100;
   struct State {
     uint8_t deck[20];       // 18 used

@@ -52,6 +52,7 @@ __host__ __device__ constexpr OcObsMasks oc_obs_masks() {
 struct EnvOvercooked {
   static constexpr bool kTurnBased = false;
   static constexpr int kNumActions = 6;
+  static constexpr bool kBinaryObs = true;  // observations are bit rows on chip
   enum : uint8_t { kNone = 0, kOnion = 1, kDish = 2, kSoup = 3 };
   struct State {
     uint8_t ax[2], ay[2];

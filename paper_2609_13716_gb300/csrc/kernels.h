@@ -30,7 +30,7 @@ struct PpoArgs {
   int64_t n_envs;
   const int32_t* perm;   // env ids grouped by teammate
   const int4* tiles;     // (perm offset, count, teammate policy, -)
-  int32_t M;             // rows per tile
+  TileCfg cfg;
   int32_t ego;
   uint32_t step0;
   int32_t T;
@@ -234,7 +234,8 @@ struct XpArgs {
   int32_t n_ego, n_tm, P, max_steps;
   int32_t ego_ids[kMaxXpIds];
   int32_t tm_ids[kMaxXpIds];
-  int32_t M, tiles_per_pair;
+  TileCfg cfg;
+  int32_t tiles_per_pair;
   uint32_t step0;
   float* returns;        // [n_pairs * P]
   int32_t* steps;        // optional
@@ -268,7 +269,7 @@ struct PolicyArgs {
   const uint8_t* obs;
   int64_t n;
   float* out;              // [n][NA+1]
-  int32_t M;
+  TileCfg cfg;
 };
 
 // Per-env launchers (defined in rollout_<env>.cu).

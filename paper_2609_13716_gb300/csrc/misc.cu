@@ -321,30 +321,47 @@ cudaError_t launch_xp_stats(const XpStatsArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// ---- standalone policy forward (test hook) ---------------------------------------------
-__global__ void __launch_bounds__(kThreads) policy_kernel(const PolicyArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
+// ---- standalone policy forward -----------------------------------------------------------
+constexpr int kPolicyThreads = 256;
+
+__global__ void __launch_bounds__(kPolicyThreads, 1) policy_kernel(const PolicyArgs a) {
+  uint8_t* const smem = tile_smem_;
   const MlpDims& m = a.b.mlp;
-  const int M = a.M;
-  const SmemLayout L = smem_layout(M, m, 0);
-  uint8_t* X = smem + L.X;
-  float* H1 = reinterpret_cast<float*>(smem + L.H1);
-  float* H2 = reinterpret_cast<float*>(smem + L.H2);
-  float* Z = reinterpret_cast<float*>(smem + L.Z);
+  const int M = a.cfg.M, tid = threadIdx.x;
+  const SmemLayout L = smem_layout(a.cfg, m, 0, 1, 0, false);
+  TileOffsets* bufs = reinterpret_cast<TileOffsets*>(smem + L.bufs);
+  MlpDims* dims = reinterpret_cast<MlpDims*>(smem + L.dims);
+  const TileOffsets to = group_offsets(L, 0);
+  const TileBufs t = tile_bufs(to);
+  const Group g{tid, kPolicyThreads, 1};
+  if (tid == 0) {
+    *bufs = to;
+    *dims = m;
+  }
+  const float* w = a.b.weights + (int64_t)a.policy * m.stride;
   const int64_t r0 = (int64_t)blockIdx.x * M;
   const int count = (int)min((int64_t)M, a.n - r0);
   const int od = m.K;
-  for (int idx = threadIdx.x; idx < M * m.KP; idx += blockDim.x) {
-    const int i = idx / m.KP, k = idx - i * m.KP;
-    X[idx] = (i < count && k < od) ? a.obs[(r0 + i) * od + k] : (uint8_t)0;
+  const uint8_t* src = a.obs + r0 * od;
+  if ((reinterpret_cast<uintptr_t>(a.obs) & 3u) == 0) {  // rows are whole words (od % 4 == 0)
+    const int wpr = od >> 2, wkp = m.KP >> 2;
+    for (int idx = tid; idx < M * wkp; idx += g.n) {
+      const int i = idx / wkp, w = idx - i * wkp;
+      reinterpret_cast<uint32_t*>(t.X)[idx] =
+          (i < count && w < wpr) ? __ldg(reinterpret_cast<const uint32_t*>(src) + i * wpr + w) : 0u;
+    }
+  } else {
+    for (int idx = tid; idx < M * m.KP; idx += g.n) {
+      const int i = idx / m.KP, k = idx - i * m.KP;
+      t.X[idx] = (i < count && k < od) ? src[i * od + k] : (uint8_t)0;
+    }
   }
-  __syncthreads();
-  mlp_tile(a.b.weights + (int64_t)a.policy * m.stride, m, X, H1, H2, Z, M,
-           reinterpret_cast<uint32_t*>(smem + L.list), count);
+  g.sync();
+  mlp_tile<false>(g.tid, g.n, g.bar, w, -1, L.dims, L.bufs, count);
   const int no = m.NA + 1;
-  for (int idx = threadIdx.x; idx < count * no; idx += blockDim.x) {
+  for (int idx = tid; idx < count * no; idx += g.n) {
     const int i = idx / no, c = idx - i * no;
-    a.out[(r0 + i) * no + c] = Z[i * m.NOP + c];
+    a.out[(r0 + i) * no + c] = t.Z[i * m.NOP + c];
   }
 }
 
@@ -353,7 +370,7 @@ cudaError_t policy_set_smem_limit(size_t bytes) {
 }
 
 cudaError_t launch_policy(const PolicyArgs& a, int grid, size_t smem, cudaStream_t s) {
-  policy_kernel<<<grid, kThreads, smem, s>>>(a);
+  policy_kernel<<<grid, kPolicyThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -1,37 +1,72 @@
-// rollout_impl.cuh -- fused persistent rollout kernels, templated on the env rules.
+// rollout_impl.cuh -- fused persistent rollout kernels on CUDA cores, templated on the env
+// rules.
 //
 // One CTA owns a tile of M envs for the whole call.  Env state lives in shared memory
 // from the first step to the last; each step the CTA builds the observations of its
 // envs in shared memory, runs the acting policies' MLPs over the tile, samples actions
 // with Philox draws, steps the envs and streams the trajectory out.  Nothing but the
 // trajectory (PPO) or the final returns (cross-play) goes back to HBM.
+//
+// Simultaneous games run the two seats at once, a group of kSeatThreads threads each with
+// its own observation and activation buffers (Group, TileBufs): their policies are
+// independent until the env step, and one seat's barriers, output layer and sampling hide
+// under the other's products.  Turn-based games run the acting seat on the whole CTA.
 #pragma once
 #include "kernels.h"
 #include "mlp_simt.cuh"
 
 namespace aht {
 
+constexpr int kTileThreads = 256;  // a CTA of the rollout kernels
+constexpr int kSeatThreads = kTileThreads / 2;
+
+// Shared memory of a CTA: the tile's states and per-env values, then `groups` sets of
+// tile buffers (TileBufs) group_stride bytes apart from g0.
 struct SmemLayout {
-  int64_t st, X, H1, H2, Z, envid, act, lp, val, alive, steps, list, total;
+  int32_t st, envid, act, lp, val, alive, steps, bufs, dims, g0, group_stride, total;
+  TileOffsets t;  // within a group
+  int32_t w3, w3_bytes;  // W3 of the CTA's policies, w3_bytes apart
 };
 
-__host__ __device__ inline SmemLayout smem_layout(int M, const MlpDims& m, int state_bytes) {
+// policies: whose W3 cfg.w3 keeps here; bits: bit rows.
+__host__ __device__ inline SmemLayout smem_layout(const TileCfg& cfg, const MlpDims& m, int state_bytes, int groups,
+                                                  int policies, bool bits) {
   SmemLayout L;
-  int64_t o = 0;
-  L.st = o;    o = align_up(o + (int64_t)M * state_bytes, 16);
-  L.X = o;     o = align_up(o + (int64_t)M * m.KP, 16);
-  L.H1 = o;    o = align_up(o + (int64_t)M * m.H0 * 4, 16);
-  L.H2 = o;    o = align_up(o + (int64_t)M * m.H1 * 4, 16);
-  L.Z = o;     o = align_up(o + (int64_t)M * m.NOP * 4, 16);
-  L.envid = o; o = align_up(o + (int64_t)M * 4, 16);
-  L.act = o;   o = align_up(o + (int64_t)M * 2, 16);
-  L.lp = o;    o = align_up(o + (int64_t)M * 4, 16);
-  L.val = o;   o = align_up(o + (int64_t)M * 4, 16);
-  L.alive = o; o = align_up(o + (int64_t)M * 4, 16);
-  L.steps = o; o = align_up(o + (int64_t)M * 4, 16);
-  L.list = o;  o = align_up(o + (m.sparse ? (int64_t)M * kSparseCap * 4 : 0), 16);
-  L.total = o;
+  auto up16 = [](int32_t x) { return (x + 15) & ~15; };
+  const int32_t M = cfg.M, ld = M + kActPad;
+  int32_t o = 0;
+  L.t.X = o;     o = up16(o + (bits ? (int32_t)M * bit_words(m.K) * 4 : (int32_t)M * m.KP));
+  const int32_t cols = m.sparse ? m.H1 : (m.K > m.H1 ? m.K : m.H1);
+  L.t.A = o;     o = up16(o + cols * ld * 4);
+  L.t.B = o;     o = up16(o + (int32_t)m.H0 * ld * 4);
+  L.t.Z = o;     o = up16(o + (int32_t)M * m.NOP * 4);
+  L.t.ks = o;    o = up16(o + (m.sparse ? 0 : (int32_t)m.K * 2));
+  L.t.list = o;  o = up16(o + (m.sparse ? (int32_t)M * kSparseCap * 4 : 0));
+  L.t.cnt = o;   o = up16(o + 8 * 4);
+  L.t.cfg = cfg;
+  L.group_stride = o;
+  o = 0;
+  L.st = o;    o = up16(o + (int32_t)M * state_bytes);
+  L.envid = o; o = up16(o + (int32_t)M * 4);
+  L.act = o;   o = up16(o + (int32_t)M * 2);
+  L.lp = o;    o = up16(o + (int32_t)M * 4);
+  L.val = o;   o = up16(o + (int32_t)M * 4);
+  L.alive = o; o = up16(o + (int32_t)M * 4);
+  L.steps = o; o = up16(o + (int32_t)M * 4);
+  L.bufs = o; o = up16(o + 2 * (int32_t)sizeof(TileOffsets));  // the groups' buffers and the dims, as
+  L.dims = o; o = up16(o + (int32_t)sizeof(MlpDims));          // mlp_tile reads them
+  L.w3 = o;
+  L.w3_bytes = cfg.w3 ? up16(m.H1 * m.NOP * 4) : 0;
+  o += policies * L.w3_bytes;
+  L.g0 = o;
+  L.total = o + groups * L.group_stride;
   return L;
+}
+
+__device__ __forceinline__ TileOffsets group_offsets(const SmemLayout& L, int group) {
+  const int d = L.g0 + group * L.group_stride;
+  return TileOffsets{L.t.X + d,  L.t.A + d,    L.t.B + d,   L.t.Z + d,
+                     L.t.ks + d, L.t.list + d, L.t.cnt + d, L.t.cfg};
 }
 
 // All of an env's state words are requested at once (one memory latency, not one per
@@ -56,85 +91,132 @@ __device__ __forceinline__ void store_state(uint32_t* __restrict__ g, int64_t n,
   for (int w = 0; w < (int)(sizeof(S) / 4); ++w) g[(int64_t)w * n + e] = p[w];
 }
 
-// Copies `count` observation rows (row i of X goes to dst row ids[i]) as 32-bit words.
-__device__ __forceinline__ void copy_obs_rows(const uint8_t* X, int KP, int count,
-                                              const int32_t* ids, uint8_t* dst, int obs_dim) {
-  const int wpr = obs_dim >> 2;
+// The tile's observation rows for `seat`, rows i < count of st (a row with alive[i] == 0 is
+// empty), zero (bit rows) or untouched (byte rows) past them.  The group synchronises at
+// the end.  Bit rows: one thread per row, the env's word writer; byte rows (LBF): the
+// row's words divided among the group's g.n / M threads per row.
+template <class Env>
+__device__ __forceinline__ void build_obs(const Group& g, const DevEnv& env, const typename Env::State* st, int seat,
+                                          int count, int M, const MlpDims& m, const TileBufs& t,
+                                          const int32_t* alive) {
+  if constexpr (Env::kBinaryObs) {
+    const int bw = bit_words(m.K);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(t.X);
+    for (int i = g.tid; i < M; i += g.n) {
+      ObsBits wr{bits + i * bw, bw};
+      if (i < count && (!alive || alive[i])) Env::obs_into(env, st[i], seat, wr);
+      else wr.clear();
+    }
+  } else {
+    const int words = m.K >> 2, per_row = g.n / M > 0 ? g.n / M : 1;
+    const int chunk = (words + per_row - 1) / per_row;
+    for (int q = g.tid; q < count * per_row; q += g.n) {
+      const int i = q / per_row, p = q - i * per_row, w0 = min(p * chunk, words);
+      if (!alive || alive[i])
+        Env::obs_words(env, st[i], seat, reinterpret_cast<uint32_t*>(t.X + i * m.KP), w0, min(w0 + chunk, words));
+    }
+  }
+  g.sync();
+}
+
+// Copies `count` observation rows (row i goes to dst row ids[i]) as 32-bit words of bytes.
+template <bool kBits>
+__device__ __forceinline__ void copy_obs_rows(const Group& g, const TileBufs& t, const MlpDims& m, int count,
+                                              const int32_t* ids, uint8_t* dst) {
+  const int wpr = m.K >> 2, bw = bit_words(m.K);
   uint32_t* d = reinterpret_cast<uint32_t*>(dst);
-  for (int idx = threadIdx.x; idx < count * wpr; idx += blockDim.x) {
+  for (int idx = g.tid; idx < count * wpr; idx += g.n) {
     const int i = idx / wpr, w = idx - i * wpr;
-    d[(int64_t)ids[i] * wpr + w] = reinterpret_cast<const uint32_t*>(X + i * KP)[w];
+    uint32_t v;
+    if constexpr (kBits) {  // four features: bit b of the nibble to byte b
+      const uint32_t nib = (reinterpret_cast<const uint32_t*>(t.X)[i * bw + (w >> 3)] >> (4 * (w & 7))) & 15u;
+      v = (nib * 0x00204081u) & 0x01010101u;
+    } else {
+      v = reinterpret_cast<const uint32_t*>(t.X + i * m.KP)[w];
+    }
+    d[(int64_t)ids[i] * wpr + w] = v;
   }
 }
 
 // ---- PPO rollout collection ------------------------------------------------------------
 template <class Env>
-__global__ void __launch_bounds__(kThreads) ppo_kernel(const PpoArgs a) {
+__global__ void __launch_bounds__(kTileThreads, 1) ppo_kernel(const PpoArgs a) {
   using State = typename Env::State;
-  extern __shared__ __align__(16) uint8_t smem[];
+  constexpr int NA = Env::kNumActions;
+  constexpr bool kBits = Env::kBinaryObs;
+  uint8_t* const smem = tile_smem_;
   const int4 tile = a.tiles[blockIdx.x];
   const int count = tile.y;
   if (count == 0) return;
-  const int M = a.M;
+  const int M = a.cfg.M;
   const MlpDims& m = a.b.mlp;
-  const SmemLayout L = smem_layout(M, m, sizeof(State));
+  const SmemLayout L = smem_layout(a.cfg, m, sizeof(State), 2, 2, kBits);
   State* st = reinterpret_cast<State*>(smem + L.st);
-  uint8_t* X = smem + L.X;
-  float* H1 = reinterpret_cast<float*>(smem + L.H1);
-  float* H2 = reinterpret_cast<float*>(smem + L.H2);
-  float* Z = reinterpret_cast<float*>(smem + L.Z);
   int32_t* envid = reinterpret_cast<int32_t*>(smem + L.envid);
   uint8_t* act = smem + L.act;
   float* lp = reinterpret_cast<float*>(smem + L.lp);
   float* val = reinterpret_cast<float*>(smem + L.val);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, seat = tid / kSeatThreads;
+  const Group g{tid - seat * kSeatThreads, kSeatThreads, 1 + seat};
+  TileOffsets* bufs = reinterpret_cast<TileOffsets*>(smem + L.bufs);
+  MlpDims* dims = reinterpret_cast<MlpDims*>(smem + L.dims);
+  const TileOffsets to = group_offsets(L, seat);
+  const TileBufs t = tile_bufs(to);
+  if (g.tid == 0) bufs[seat] = to;
+  if (tid == 0) *dims = m;
   const int64_t N = a.n_envs;
   const int od = a.b.env.obs_dim;
+  const TrajPtrs& traj = seat == 0 ? a.traj : a.traj1;  // this seat's learner fields
 
-  for (int i = tid; i < M; i += blockDim.x) {
-    if (i < count) {
-      const int env = a.perm[tile.x + i];
-      envid[i] = env;
-      load_state(a.state, N, env, st[i]);
-    }
-    uint32_t* row = reinterpret_cast<uint32_t*>(X + i * m.KP);
-    for (int w = 0; w < (m.KP >> 2); ++w) row[w] = 0u;  // padding columns stay zero
+  for (int i = tid; i < count; i += blockDim.x) {
+    const int env = a.perm[tile.x + i];
+    envid[i] = env;
+    load_state(a.state, N, env, st[i]);
   }
+  if (!kBits)  // padding columns and the rows past count stay zero
+    for (int i = g.tid; i < M * (m.KP >> 2); i += g.n) reinterpret_cast<uint32_t*>(t.X)[i] = 0u;
+  const float* w_pol = a.b.weights + (int64_t)(seat == 0 ? a.ego : tile.z) * m.stride;
+  const int o_w3 = a.cfg.w3 ? L.w3 + seat * L.w3_bytes : -1;
+  if (o_w3 >= 0) load_w3(g, w_pol, m, reinterpret_cast<float*>(smem + o_w3));
   __syncthreads();
-  const float* w_pol[2] = {a.b.weights + (int64_t)a.ego * m.stride,
-                           a.b.weights + (int64_t)tile.z * m.stride};
 
-  for (int t = 0; t < a.T; ++t) {
-    const uint32_t gt = a.step0 + (uint32_t)t;
-    for (int seat = 0; seat < 2; ++seat) {
-      for (int i = tid; i < count; i += blockDim.x) Env::obs(a.b.env, st[i], seat, X + i * m.KP);
-      __syncthreads();
-      if (seat == 0 && a.traj.obs)
-        copy_obs_rows(X, m.KP, count, envid, a.traj.obs + (int64_t)t * N * od, od);
-      if (seat == 1 && a.traj1.obs)
-        copy_obs_rows(X, m.KP, count, envid, a.traj1.obs + (int64_t)t * N * od, od);
-      mlp_tile(w_pol[seat], m, X, H1, H2, Z, M, reinterpret_cast<uint32_t*>(smem + L.list), count);
-      for (int i = tid; i < count; i += blockDim.x) {
-        const float u = u01(draw0(a.b.key, (uint32_t)envid[i], gt, kStreamAct0 + seat));
-        float logp;
-        const int ai = sample_row(Z + i * m.NOP, m.NA, 0xFFFFFFFFu >> (32 - m.NA), u, logp);
-        act[i * 2 + seat] = (uint8_t)ai;
-        if (seat == 0) {
-          lp[i] = logp;
-          val[i] = Z[i * m.NOP + m.NA];
-        } else {
-          const int64_t o = (int64_t)t * N + envid[i];
-          if (a.traj1.logp) a.traj1.logp[o] = logp;
-          if (a.traj1.values) a.traj1.values[o] = Z[i * m.NOP + m.NA];
-        }
-      }
-      __syncthreads();
+  // Steps 0..T-1, then the bootstrap value V_T of the state after the last step where asked.
+  for (int s = 0; s <= a.T; ++s) {
+    const bool boot = s == a.T;
+    const uint32_t gt = a.step0 + (uint32_t)s;
+    if (!boot || traj.last_value) {
+      build_obs<Env>(g, a.b.env, st, seat, count, M, m, t, nullptr);
+      if (!boot && traj.obs) copy_obs_rows<kBits>(g, t, m, count, envid, traj.obs + (int64_t)s * N * od);
+      mlp_tile<kBits>(g.tid, g.n, g.bar, w_pol, o_w3, L.dims, L.bufs + seat * (int)sizeof(TileOffsets), count);
     }
+    if (boot) {
+      if (traj.last_value)
+        for (int i = g.tid; i < count; i += g.n) traj.last_value[envid[i]] = t.Z[i * m.NOP + NA];
+      break;
+    }
+    for (int i = g.tid; i < count; i += g.n) {
+      const float u = u01(draw0(a.b.key, (uint32_t)envid[i], gt, kStreamAct0 + seat));
+      float z[NA];
+#pragma unroll
+      for (int o = 0; o < NA; ++o) z[o] = t.Z[i * m.NOP + o];
+      float logp;
+      act[i * 2 + seat] = (uint8_t)sample_k<NA>(z, 0xFFFFFFFFu >> (32 - NA), u, logp);
+      const float v = t.Z[i * m.NOP + NA];
+      if (seat == 0) {
+        lp[i] = logp;
+        val[i] = v;
+      } else {
+        const int64_t o = (int64_t)s * N + envid[i];
+        if (traj.logp) traj.logp[o] = logp;
+        if (traj.values) traj.values[o] = v;
+      }
+    }
+    __syncthreads();
     for (int i = tid; i < count; i += blockDim.x) {
       const int env = envid[i];
       float r0, r1, team;
       const int done = Env::step(a.b.env, st[i], act[2 * i], act[2 * i + 1], r0, r1, team);
-      const int64_t o = (int64_t)t * N + env;
+      const int64_t o = (int64_t)s * N + env;
       if (a.traj.actions) a.traj.actions[o] = act[2 * i];
       if (a.traj.tm_actions) a.traj.tm_actions[o] = act[2 * i + 1];
       if (a.traj.logp) a.traj.logp[o] = lp[i];
@@ -152,40 +234,32 @@ __global__ void __launch_bounds__(kThreads) ppo_kernel(const PpoArgs a) {
     }
     __syncthreads();
   }
-  // Bootstrap value V_T of the state after the last step.
-  if (a.traj.last_value) {
-    for (int i = tid; i < count; i += blockDim.x) Env::obs(a.b.env, st[i], 0, X + i * m.KP);
-    __syncthreads();
-    mlp_tile(w_pol[0], m, X, H1, H2, Z, M, reinterpret_cast<uint32_t*>(smem + L.list), count);
-    for (int i = tid; i < count; i += blockDim.x) a.traj.last_value[envid[i]] = Z[i * m.NOP + m.NA];
-    __syncthreads();
-  }
-  if (a.traj1.last_value) {  // seat 1's V_T (IPPO)
-    for (int i = tid; i < count; i += blockDim.x) Env::obs(a.b.env, st[i], 1, X + i * m.KP);
-    __syncthreads();
-    mlp_tile(w_pol[1], m, X, H1, H2, Z, M, reinterpret_cast<uint32_t*>(smem + L.list), count);
-    for (int i = tid; i < count; i += blockDim.x) a.traj1.last_value[envid[i]] = Z[i * m.NOP + m.NA];
-  }
   for (int i = tid; i < count; i += blockDim.x) store_state(a.state, N, envid[i], st[i]);
 }
 
 // ---- cross-play evaluation --------------------------------------------------------------
 template <class Env>
-__global__ void __launch_bounds__(kThreads) xplay_kernel(const XpArgs a) {
+__global__ void __launch_bounds__(kTileThreads, 1) xplay_kernel(const XpArgs a) {
   using State = typename Env::State;
-  extern __shared__ __align__(16) uint8_t smem[];
-  const int M = a.M;
+  constexpr int NA = Env::kNumActions;
+  constexpr bool kBits = Env::kBinaryObs, kTurn = Env::kTurnBased;
+  uint8_t* const smem = tile_smem_;
+  const int M = a.cfg.M;
   const MlpDims& m = a.b.mlp;
-  const SmemLayout L = smem_layout(M, m, sizeof(State));
+  const SmemLayout L = smem_layout(a.cfg, m, sizeof(State), kTurn ? 1 : 2, 2, kBits);
   State* st = reinterpret_cast<State*>(smem + L.st);
-  uint8_t* X = smem + L.X;
-  float* H1 = reinterpret_cast<float*>(smem + L.H1);
-  float* H2 = reinterpret_cast<float*>(smem + L.H2);
-  float* Z = reinterpret_cast<float*>(smem + L.Z);
   uint8_t* act = smem + L.act;
   int32_t* alive = reinterpret_cast<int32_t*>(smem + L.alive);
   int32_t* nsteps = reinterpret_cast<int32_t*>(smem + L.steps);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, half = tid / kSeatThreads;
+  const Group g = kTurn ? Group{tid, kTileThreads, 1} : Group{tid - half * kSeatThreads, kSeatThreads, 1 + half};
+  TileOffsets* bufs = reinterpret_cast<TileOffsets*>(smem + L.bufs);
+  MlpDims* dims = reinterpret_cast<MlpDims*>(smem + L.dims);
+  const int set = kTurn ? 0 : half;
+  const TileOffsets to = group_offsets(L, set);
+  const TileBufs t = tile_bufs(to);
+  if (g.tid == 0) bufs[set] = to;
+  if (tid == 0) *dims = m;
 
   const int pair = blockIdx.x / a.tiles_per_pair;
   const int first = (blockIdx.x - pair * a.tiles_per_pair) * M;
@@ -199,34 +273,37 @@ __global__ void __launch_bounds__(kThreads) xplay_kernel(const XpArgs a) {
     if (i < count) Env::reset(a.b.env, a.b.key, (uint32_t)(e0 + i), a.step0, st[i]);
     alive[i] = i < count;
     nsteps[i] = 0;
-    uint32_t* row = reinterpret_cast<uint32_t*>(X + i * m.KP);
-    for (int w = 0; w < (m.KP >> 2); ++w) row[w] = 0u;
   }
+  if (!kBits)
+    for (int i = g.tid; i < M * (m.KP >> 2); i += g.n) reinterpret_cast<uint32_t*>(t.X)[i] = 0u;
+  const bool w3s = a.cfg.w3 != 0;
+  for (int p = 0; w3s && p < 2; ++p)
+    load_w3(Group{tid, kTileThreads, 0}, w_pol[p], m, reinterpret_cast<float*>(smem + L.w3 + p * L.w3_bytes));
   __syncthreads();
 
   for (int s = 0; s < a.max_steps; ++s) {
     if (!__syncthreads_or(tid < count && alive[tid])) break;
     const uint32_t gt = a.step0 + (uint32_t)s;
-    const int actor = Env::kTurnBased ? (s & 1) : -1;
-    for (int seat = 0; seat < 2; ++seat) {
-      if (actor >= 0 && seat != actor) continue;
-      for (int i = tid; i < count; i += blockDim.x)
-        if (alive[i]) Env::obs(a.b.env, st[i], seat, X + i * m.KP);
-      __syncthreads();
-      mlp_tile(w_pol[seat], m, X, H1, H2, Z, M, reinterpret_cast<uint32_t*>(smem + L.list), count);
-      for (int i = tid; i < count; i += blockDim.x) {
-        if (!alive[i]) continue;
-        uint32_t legal = 0xFFFFFFFFu >> (32 - m.NA);
-        if (Env::kTurnBased) {
-          legal = Env::legal(st[i]);
-          if (Env::actor(st[i]) != seat) atomicOr(a.b.status, kStatusActorMismatch);
-        }
-        const float u = u01(draw0(a.b.key, (uint32_t)(e0 + i), gt, kStreamAct0 + seat));
-        float logp;
-        act[i * 2 + seat] = (uint8_t)sample_row(Z + i * m.NOP, m.NA, legal, u, logp);
+    const int actor = kTurn ? (s & 1) : -1;
+    const int seat = kTurn ? actor : half;
+    build_obs<Env>(g, a.b.env, st, seat, count, M, m, t, alive);
+    mlp_tile<kBits>(g.tid, g.n, g.bar, seat ? w_pol[1] : w_pol[0], w3s ? L.w3 + seat * L.w3_bytes : -1, L.dims,
+                    L.bufs + set * (int)sizeof(TileOffsets), count);
+    for (int i = g.tid; i < count; i += g.n) {
+      if (!alive[i]) continue;
+      uint32_t legal = 0xFFFFFFFFu >> (32 - NA);
+      if (kTurn) {
+        legal = Env::legal(st[i]);
+        if (Env::actor(st[i]) != seat) atomicOr(a.b.status, kStatusActorMismatch);
       }
-      __syncthreads();
+      const float u = u01(draw0(a.b.key, (uint32_t)(e0 + i), gt, kStreamAct0 + seat));
+      float z[NA];
+#pragma unroll
+      for (int o = 0; o < NA; ++o) z[o] = t.Z[i * m.NOP + o];
+      float logp;
+      act[i * 2 + seat] = (uint8_t)sample_k<NA>(z, legal, u, logp);
     }
+    __syncthreads();
     for (int i = tid; i < count; i += blockDim.x) {
       const int64_t e = e0 + i;
       // (the host pre-fills the optional action record with 255 = no action)
@@ -302,11 +379,11 @@ template <class Env>
 struct Launch {
   using State = typename Env::State;
   static cudaError_t ppo(const PpoArgs& a, int grid, size_t smem, cudaStream_t s) {
-    ppo_kernel<Env><<<grid, kThreads, smem, s>>>(a);
+    ppo_kernel<Env><<<grid, kTileThreads, smem, s>>>(a);
     return cudaGetLastError();
   }
   static cudaError_t xplay(const XpArgs& a, int grid, size_t smem, cudaStream_t s) {
-    xplay_kernel<Env><<<grid, kThreads, smem, s>>>(a);
+    xplay_kernel<Env><<<grid, kTileThreads, smem, s>>>(a);
     return cudaGetLastError();
   }
   static cudaError_t forced(const ForcedArgs& a, cudaStream_t s) {
@@ -340,8 +417,8 @@ struct Launch {
   cudaError_t name##_set_smem_limit(size_t b) { return Launch<EnvT>::smem_limit(b); }            \
   int name##_occupancy(int which, size_t sm) {                                                 \
     int n = 0;                                                                                 \
-    if (which == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ppo_kernel<EnvT>, kThreads, sm); \
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, xplay_kernel<EnvT>, kThreads, sm);  \
+    if (which == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ppo_kernel<EnvT>, kTileThreads, sm); \
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, xplay_kernel<EnvT>, kTileThreads, sm);  \
     cudaGetLastError();                                                                        \
     return n;                                                                                  \
   }
