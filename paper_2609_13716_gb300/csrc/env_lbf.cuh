@@ -205,6 +205,23 @@ struct EnvLbf {
     put(s1 ? s.ax[1] : s.ax[0], s1 ? s.ay[1] : s.ay[0], (uint32_t)(s1 ? s.al[1] : s.al[0]));
   }
 
+  // Turns seat 0's row of state s (as obs_words writes it) into that of its successor n, whose
+  // foods are s's minus the ones eaten, or new ones when `fresh` (a reset): the cells that s's
+  // agents and gone foods leave become empty, then n's agents and new foods are put down.
+  __device__ static void move_words(const DevEnv& d, const State& s, const State& n, bool fresh, uint32_t* w) {
+    auto cell = [&](int x, int y) { return y * d.width + x; };
+    w[cell(s.ax[0], s.ay[0])] = 0x01000000u;
+    w[cell(s.ax[1], s.ay[1])] = 0x01000000u;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (!((s.eaten >> k) & 1u) && (fresh || ((n.eaten >> k) & 1u))) w[cell(s.fx[k], s.fy[k])] = 0x01000000u;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (fresh && !((n.eaten >> k) & 1u)) w[cell(n.fx[k], n.fy[k])] = (uint32_t)n.fl[k] << 16;
+    w[cell(n.ax[1], n.ay[1])] = (uint32_t)n.al[1] << 8;
+    w[cell(n.ax[0], n.ay[0])] = (uint32_t)n.al[0];
+  }
+
   // Rule-based teammate k in seat 1 (the LBF heuristic suite: Greedy criteria 0..4,
   // Sequential orderings 5..10, Entitled 11): the cell to go for, then load when there,
   // else a step along the axis with the larger remaining distance (ties: x), else along

@@ -3,8 +3,8 @@
 //
 // One CTA owns a tile of up to 128 envs that share a teammate policy, for all T steps.
 // Per step and agent (ego = seat 0, teammate = seat 1):
-//   obs (u8, shared memory, a constant 1 after the last feature) -> A operand in tensor
-//       memory as bf16 (exact: small integers)
+//   obs (u8 rows kept in shared memory, a constant 1 after the last feature) -> A operand in
+//       tensor memory as bf16 (exact: small integers)
 //   L1 (tensor cores): D = [o 1] [W1 b1]^T      (M = 128 envs, N = hidden0, K = KP)
 //   epilogue 1: r1 = 1 / (1 + exp(2 D)) split r1 = hi + lo (two bf16) into tensor memory;
 //       tanh(D) = 1 - 2 r1, and the block's W2, b2 hold -2 W2 and b2 + W2 1, so L2 sees
@@ -23,18 +23,24 @@
 // sampling) run concurrently, four warps per SM sub-partition.  There is no MMA warp
 // (sixteen warps keep 128 registers a thread): once a group's operand is in tensor memory
 // (a group barrier), its first thread issues the layer's MMAs and commits them to the
-// group's accumulator barrier.  The groups share one observation buffer: the teammate's
-// rows are built first, and once they are in tensor memory the buffer passes to the ego
-// (an mbarrier).  Both groups meet twice per step on a named barrier that also ORs their
-// error flags: once both actions exist (then the ego group's first half steps the envs
-// while, for gathered tiles, the teammate group and the ego's second half write the ego's
-// rows to the trajectory) and once the new state is in shared memory.  Every mbarrier wait
+// group's accumulator barrier.  The observation rows (the ego's view) stay in shared memory
+// across steps: the thread that steps an env moves the changed cells of its row, at most ten
+// words, and both groups read the rows, the teammate with the level channels swapped.  The
+// rows go to the trajectory by a bulk copy (contiguous tiles) or by the teammate group before
+// its own chain starts (gathered ones).  Both groups meet twice per step
+// on a named barrier that also ORs their error flags: once both actions exist (then the ego
+// group's first half steps the envs) and once the new state and its rows are in shared
+// memory.  What bounds it is the length of a step's chain, not a pipe (issue slots half
+// busy): building a row anew for each agent in turn, through one buffer, made LBF 7x7
+// collection 16384 x 128 1.19 ms, now 1.09 (64 envs x 50 steps 373 -> 318 us).  Every mbarrier wait
 // is bounded (2 s): on expiry the CTA records kStatusTimeout, stops, waits (bounded) for
 // its own MMAs, frees tensor memory and exits.
 //
 // Tensor memory (512 columns): agent a uses columns [256a, 256a + 128) for its A operand
 // (X, then hi|lo of h1) and [256a + 128, 256a + 256) for its fp32 accumulator.
 #pragma once
+#include <type_traits>
+
 #include "rollout_tc.cuh"
 
 namespace aht {
@@ -43,6 +49,7 @@ constexpr int kT2Group = 256;     // threads per agent group
 constexpr int kT2Threads = 512;   // both groups
 constexpr int kT2AllBar = 1;      // named barrier ids: both groups (OR of the error flags)
 constexpr int kT2GroupBar = 2;    // 2 + g: group g
+constexpr int kT2StaggerBar = 15; // both groups: the ego arrives, the teammate waits
 constexpr int kT2PairBar = 4;     // 4 + 4 g + q: warps 8 g + q and 8 g + q + 4 (rows 32 q ..)
 
 // kXp: cross-play instead of collection -- a tile is up to 128 envs of one pair (ego i,
@@ -61,7 +68,6 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ __align__(8) uint64_t acc_bar[4];     // [2*agent + layer], tcgen05.commit
   __shared__ __align__(8) uint64_t wload_bar[2], drain_bar[2];  // per agent
-  __shared__ __align__(8) uint64_t buf_free;       // teammate rows in tensor memory (256)
   __shared__ __align__(8) uint64_t never_bar;      // test hook: nothing arrives on it
   __shared__ uint32_t tmem_slot;
   const TcDims& d = a.tc;
@@ -78,7 +84,6 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
       tc::mbar_init(&wload_bar[i], 1);
       tc::mbar_init(&drain_bar[i], 1);
     }
-    tc::mbar_init(&buf_free, kT2Group);
     tc::mbar_init(&never_bar, 1);
     tc::mbar_init_fence();
     // the ego's policy block -> shared memory, waited for by the ego group (collection:
@@ -130,10 +135,11 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
   const int chunks = d.KP / 16;
   const int split = (chunks + 1) / 2;
   const int my_c0 = half ? split : 0, my_c1 = half ? chunks : split;
-  const int my_w0 = min(4 * my_c0, cells), my_w1 = min(4 * my_c1, cells);
   const bool boot1 = kIppo && tm_pol >= 0 && a.traj1.last_value != nullptr;  // seat 1's V_T
   const bool with_boot = !kXp && (a.traj.last_value != nullptr || boot1);
-  const bool obs_copy = kGather && a.traj.obs != nullptr;  // 12 warps store the rows during the step
+  const bool obs_copy = kGather && a.traj.obs != nullptr;  // the warps store gathered rows
+  // one-step launches without a V_T never move the rows: they leave while the envs step
+  const bool late_copy = kGather && a.g.resample && !with_boot && obs_copy;
 
   uint8_t* const sW0 = smem;                                                // policy blocks
   uint8_t* const sObs = smem + 2 * d.pol_bytes;                             // [128][obs_dim] u8
@@ -141,7 +147,6 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
   uint8_t* act1s = reinterpret_cast<uint8_t*>(st) + align_up(128 * sizeof(State), 16);  // [128]
   float* zpart = reinterpret_cast<float*>(act1s + 128);                     // [2][2][128][8]
 
-  for (int i = tid; i < 32 * od; i += blockDim.x) reinterpret_cast<uint32_t*>(sObs)[i] = 0u;
   if (tid < count) {
     if constexpr (kXp) Env::reset(a.b.env, a.b.key, (uint32_t)(env0 + tid), a.step0, st[tid]);
     else load_state(a.state, N, env_of(tid), st[tid]);
@@ -150,6 +155,19 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  {  // the ego's rows of the first state, a quarter of a row per thread (rows past count: zero)
+    const int quarter = 2 * grp + half, per = (cells + 3) / 4;
+    const int w0 = min(quarter * per, cells), w1 = min(w0 + per, cells);
+    uint32_t* roww = reinterpret_cast<uint32_t*>(sObs + row * od);
+    if (row < count) {
+      const State s0 = st[row];
+      Env::obs_words(a.b.env, s0, 0, roww, w0, w1);
+    } else {
+      for (int w = w0; w < w1; ++w) roww[w] = 0u;
+    }
+  }
+  if (!kGather) tc::fence_proxy_async();  // (the bulk copy engine reads contiguous tiles' rows)
+  __syncthreads();
 
   {
     const int ag = grp;  // the agent this thread works for
@@ -204,10 +222,6 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
       bad = __any_sync(0xFFFFFFFFu, bad);  // warp-uniform: tensor-memory loads are collective
       tc::fence_after_sync();
     };
-    auto wait_bar = [&](uint64_t* bar, uint32_t parity) {
-      if (!bad && !tc::mbar_wait(bar, parity)) bad = true;
-      bad = __any_sync(0xFFFFFFFFu, bad);
-    };
     // both groups; every thread leaves with the OR of the error flags
     auto sync_all = [&]() {
       bad = tc::bar_or(kT2AllBar, kT2Threads, bad);
@@ -217,25 +231,37 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
     const uint8_t* const pol_block = sW0 + (size_t)ag * d.pol_bytes;
     const uint32_t P = tmem + (uint32_t)(ag * 256) + lane_base, Q = P + 128;
 
-    // observation (this thread's half row, built in shared memory) -> bf16 A operand of
-    // L1 in tensor memory; feature obs_dim is the constant 1 that carries b1
-    auto obs_x = [&](const State& s) {
-      uint32_t* roww = reinterpret_cast<uint32_t*>(sObs + row * od);
-      if (row < count) Env::obs_words(a.b.env, s, ag, roww, my_w0, my_w1);
-      for (int c = my_c0; c < my_c1; ++c) {
+    // this thread's half of its row (the ego's view, in shared memory) -> bf16 A operand of
+    // L1 in tensor memory; the teammate sees the two level channels (bytes 0 and 1)
+    // swapped.  Feature obs_dim is the constant 1 that carries b1.
+    const uint32_t sel01 = ag == 0 ? 0x4140u : 0x4041u;
+    auto obs_x = [&]() {
+      const uint32_t* roww = reinterpret_cast<const uint32_t*>(sObs + row * od);
+      const int c_full = min(my_c1, cells >> 2);  // chunks of four cells; then the row's end
+      auto expand = [&](int c, const uint32_t (&w4)[4]) {
+        uint32_t v[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          v[2 * j] = tc::small_bytes_to_bf16x2(w4[j], sel01);
+          v[2 * j + 1] = tc::small_bytes_to_bf16x2(w4[j], 0x4342u);
+        }
+        tc::st_x8(P + 8 * c, v);
+      };
+#pragma unroll 1
+      for (int c = my_c0; c < c_full; ++c) {
+        uint32_t w4[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w4[j] = roww[4 * c + j];
+        expand(c, w4);
+      }
+      for (int c = max(my_c0, c_full); c < my_c1; ++c) {
         uint32_t w4[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int w = 4 * c + j;
-          w4[j] = w < cells ? roww[w] : (w == cells ? 1u : 0u);
+          w4[j] = w < cells ? roww[w] : (w == cells ? (ag == 0 ? 1u : 0x100u) : 0u);
         }
-        uint32_t v[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          v[2 * j] = tc::bytes_to_bf16x2(w4[j], 0);
-          v[2 * j + 1] = tc::bytes_to_bf16x2(w4[j], 2);
-        }
-        tc::st_x8(P + 8 * c, v);
+        expand(c, w4);
       }
       tc::wait_st();
     };
@@ -362,23 +388,41 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
         for (uint32_t w = tid; w < bytes / 4; w += kT2Group) d32[w] = src[w];
       }
     };
-    // gathered tiles: the ego's rows -> their envs' trajectory rows, while the ego group's
-    // first half steps the envs: the 12 warps of the teammate group and of the ego's
-    // second half take the tile's count x cells words in turn (consecutive lanes,
-    // consecutive words of a row; row = word / cells by a reciprocal multiply, exact for
-    // fewer than 2^16 words)
-    const uint32_t cells_rcp = 0xFFFFFFFFu / (uint32_t)cells + 1u;
-    auto copy_rows_gathered = [&](int t, int cw) {
-      constexpr int kCopyWarps = 12;
+    // gathered tiles: the ego's rows -> their envs' trajectory rows by the teammate group,
+    // before its own L1 operand: the tile's count x cells words in turn (consecutive lanes,
+    // consecutive words of a row; row = word / cells by a reciprocal multiply, exact for fewer
+    // than 2^16 words).  The teammate's chain then runs ~2.4 K cycles behind the ego's, so one
+    // group's epilogues fall under the other's products, and the ego's spare time at the end
+    // goes to its trajectory fields.  (C2 1.09 ms; the rows copied by both groups while L1 or
+    // L2 runs, which keeps the chains in phase or slows the epilogues, 1.14-1.24; a warp per
+    // row 1.11.)
+    auto copy_rows_gathered = [&](int t, int cw, auto warps) {  // warp cw of `warps`
+      constexpr int n_warps = decltype(warps)::value;
       uint32_t* const base = reinterpret_cast<uint32_t*>(a.traj.obs + (int64_t)t * N * od);
       const uint32_t* const src = reinterpret_cast<const uint32_t*>(sObs);
       const int total = count * cells;
+      const uint32_t cells_rcp = 0xFFFFFFFFu / (uint32_t)cells + 1u;
 #pragma unroll 4
-      for (int f = cw * 32 + lane; f < total; f += kCopyWarps * 32) {
+      for (int f = cw * 32 + lane; f < total; f += n_warps * 32) {
         const int r = (int)__umulhi((uint32_t)f, cells_rcp);
         base[(int64_t)rowenv[r] * cells + (f - r * cells)] = src[f];
       }
     };
+    // the rows of this step's state that the teammate group's warps store before its operand
+    auto copy_rows = [&](int t) {
+      if (obs_copy && !late_copy) copy_rows_gathered(t, warp - 8, std::integral_constant<int, 8>());
+      if (kIppo && a.traj1.obs) {  // seat 1's rows, a contiguous block
+        const uint32_t* const src = reinterpret_cast<const uint32_t*>(sObs);
+        uint32_t* const dst = reinterpret_cast<uint32_t*>(a.traj1.obs + ((int64_t)t * N + env0) * od);
+        for (int f = tid - kT2Group; f < count * cells; f += kT2Group) dst[f] = Env::other_seat_word(src[f]);
+      }
+    };
+
+    // contiguous tiles: with 128-wide layers the teammate waits until the ego's L1 is issued,
+    // so that the two chains' products and epilogues alternate (collection 5000 x 64 561 -> 487
+    // us, IPPO 1.15 -> 1.05 ms, cross-play 8 x 16 x 128 0.97 -> 0.86); 64-wide ones, whose
+    // epilogues are half as long, run in phase (cross-play 8 x 16 x 256 1.45 ms, staggered 1.63)
+    const bool stagger = !kGather && d.H0 > 64;
 
     // Steps 0..T-1, then (if requested) the ego's V_T of the state after the last step.
     const int n_steps = kXp ? a.xp.max_steps : a.T;
@@ -397,17 +441,18 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
       auto draw_action = [&]() {
         if (sampler) u_act = u01(draw0(a.b.key, (uint32_t)my_env, gt, kStreamAct0 + ag));
       };
-      const State s = st[row];  // register copy for this step (rows past count are never used)
       float z[16];
       int act0 = 0;
-      float lp0 = 0.f, val0 = 0.f;
       if (ag == 1) {
         // ---------------------------- teammate group -------------------------------
         const bool run = (!boot || boot1) && !tm_rule;
-        if (run) obs_x(s);
-        tc::mbar_arrive(&buf_free);  // its rows are in tensor memory: the buffer is the ego's
+        if (!boot) copy_rows(t);
+        if (stagger) tc::bar_sync(kT2StaggerBar, kT2Threads);
         if (run) {
+          obs_x();
           issue(0);
+        }
+        if (run) {
           draw_action();
           wait_acc(0, par);
           if (!bad) epilogue1();
@@ -418,7 +463,7 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
         pair_sync();
         if (sampler) {
           if (tm_rule) {
-            act1s[row] = (uint8_t)Env::heuristic(a.b.env, st[row], -1 - tm_pol);  // st[row] == s
+            act1s[row] = (uint8_t)Env::heuristic(a.b.env, st[row], -1 - tm_pol);
           } else {
             logits(z);
             dbg_store(t, z);
@@ -436,13 +481,11 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
         }
       } else {
         // ------------------------------- ego group ---------------------------------
-        wait_bar(&buf_free, par);
-        obs_x(s);
-        // contiguous tiles: the rows (ordinary stores) are read by the bulk copy engine
-        if (!kGather && !boot && a.traj.obs) tc::fence_proxy_async();
-        issue(0);  // (its group barrier also orders the rows before the copy)
-        draw_action();
+        obs_x();
+        issue(0);
+        if (stagger) tc::bar_arrive(kT2StaggerBar, kT2Threads);
         if (!kGather && !boot && a.traj.obs) copy_rows_contiguous(t);
+        draw_action();
         if (t == a.dbg_expire_step) {  // test hook: an accumulator wait that never completes
           if (!bad && !tc::mbar_wait(&never_bar, 0, a.dbg_expire_ns)) bad = true;
           bad = __any_sync(0xFFFFFFFFu, bad);
@@ -461,13 +504,22 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
         } else if (sampler) {
           logits(z);
           dbg_store(t, z);
+          float lp0;
           act0 = sample_k<NA>(z, 0xFFFFFFFFu >> (32 - NA), u_act, lp0);
-          val0 = z[NA];
+          if constexpr (!kXp) {  // while the teammate's chain, which starts later, finishes
+            const int64_t o = (int64_t)t * N + my_env;
+            if (a.traj.actions) a.traj.actions[o] = (uint8_t)act0;
+            if (a.traj.logp) a.traj.logp[o] = lp0;
+            if (a.traj.values) a.traj.values[o] = z[NA];
+            if (kIppo && a.traj1.tm_actions) a.traj1.tm_actions[o] = (uint8_t)act0;
+          }
         }
       }
-      if (sync_all() || boot) break;  // both actions exist
+      if (tid == 0 && bulk_obs) tc::bulk_wait_read();  // the rows may change
+      if (sync_all() || boot) break;                    // both actions exist, the rows are stored
       bool stayed = false;            // per-episode gather: the env keeps its teammate
       if (kXp && ag == 0 && half == 0 && row < count && alive) {
+        const State s = st[row];
         State s2 = s;
         const int act1 = act1s[row];
         if (a.xp.actions) {
@@ -485,7 +537,9 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
           if (done) alive = false;
         }
         st[row] = s2;
+        Env::move_words(a.b.env, s, s2, false, reinterpret_cast<uint32_t*>(sObs + row * od));
       } else if (!kXp && ag == 0 && half == 0 && row < count) {
+        const State s = st[row];
         State s2 = s;
         const int act1 = act1s[row];
         const int64_t env = my_env;
@@ -496,15 +550,11 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
         float r0, r1, team;
         const int done = Env::step(a.b.env, s2, act0, act1, r0, r1, team);
         const int64_t o = (int64_t)t * N + env;
-        if (a.traj.actions) a.traj.actions[o] = (uint8_t)act0;
         if (a.traj.tm_actions) a.traj.tm_actions[o] = (uint8_t)act1;
-        if (a.traj.logp) a.traj.logp[o] = lp0;
-        if (a.traj.values) a.traj.values[o] = val0;
         if (a.traj.rewards) a.traj.rewards[o] = team;
         if (a.traj.dones) a.traj.dones[o] = (uint8_t)(done > 0);
         if constexpr (kIppo) {  // seat 1's learner fields
           if (a.traj1.actions) a.traj1.actions[o] = (uint8_t)act1;
-          if (a.traj1.tm_actions) a.traj1.tm_actions[o] = (uint8_t)act0;
           if (a.traj1.rewards) a.traj1.rewards[o] = team;
           if (a.traj1.dones) a.traj1.dones[o] = (uint8_t)(done > 0);
         }
@@ -523,20 +573,15 @@ __global__ void __launch_bounds__(kT2Threads, 1) ppo2_tc_kernel(const PpoTcArgs 
           stayed = done <= 0;
         }
         st[row] = s2;
+        if (!late_copy) Env::move_words(a.b.env, s, s2, done > 0, reinterpret_cast<uint32_t*>(sObs + row * od));
+        if (!kGather) tc::fence_proxy_async();
       }
       if (kGather && a.g.resample && ag == 0 && half == 0) {
         const unsigned m = __ballot_sync(0xFFFFFFFFu, stayed);
         if (lane == 0 && m) atomicAdd(&a.g.hist_next[g_k], __popc(m));
       }
-      if (obs_copy && (ag == 1 || half == 1)) copy_rows_gathered(t, ag == 1 ? warp - 8 : warp + 4);
-      if (kIppo && a.traj1.obs && (ag == 1 || half == 1)) {  // seat 1's rows, a contiguous block
-        const int cw = ag == 1 ? warp - 8 : warp + 4;
-        const uint32_t* const src = reinterpret_cast<const uint32_t*>(sObs);
-        uint32_t* const dst = reinterpret_cast<uint32_t*>(a.traj1.obs + ((int64_t)t * N + env0) * od);
-        for (int f = cw * 32 + lane; f < count * cells; f += 12 * 32) dst[f] = Env::other_seat_word(src[f]);
-      }
-      if (tid == 0 && bulk_obs) tc::bulk_wait_read();  // the rows may be rebuilt
-      if (sync_all()) break;                            // the new state is in place
+      if (late_copy && (ag == 1 || half == 1)) copy_rows_gathered(t, ag == 1 ? warp - 8 : warp + 4, std::integral_constant<int, 12>());
+      if (sync_all()) break;  // the new state and its rows are in place
     }
     if (tid == 0 && bulk_obs) tc::bulk_wait_all();
     if (bad) {

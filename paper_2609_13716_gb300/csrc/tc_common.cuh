@@ -203,6 +203,11 @@ __device__ __forceinline__ void bar_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// Arrival at a named barrier of `count` threads without waiting (the others bar_sync).
+__device__ __forceinline__ void bar_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
 // Named barrier over `count` threads with an OR reduction of `pred` (all get the OR).
 __device__ __forceinline__ bool bar_or(int id, int count, bool pred) {
   uint32_t r;
@@ -319,6 +324,18 @@ __device__ __forceinline__ uint32_t bytes_to_bf16x2(uint32_t w, int first) {
                    two23),
             f0, f1);
   return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+}
+
+// Two bytes below 128 of a 32-bit word as a packed bf16x2 in two instructions: the bf16 bits
+// 0x4300 | b are 128 + b (its unit in the last place there is 1), so one byte permutation
+// makes both and one packed subtraction of 128 leaves b exactly.  sel: the byte indexes,
+// (second << 8 | first) in its low nibbles, 4 in the others (0x4140: bytes 0 and 1).
+__device__ __forceinline__ uint32_t small_bytes_to_bf16x2(uint32_t w, uint32_t sel) {
+  uint32_t r;
+  // result bytes, low to high: b[first], 0x43, b[second], 0x43
+  const uint32_t biased = __byte_perm(w, 0x43434343u, sel);
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(biased), "r"(0x43004300u));
+  return r;
 }
 
 // 2 / ln 2 in each half of a pair: x (2 / ln 2) is the exponent of 2 that gives exp(2x).
