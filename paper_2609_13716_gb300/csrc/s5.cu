@@ -76,6 +76,7 @@ namespace {
 // (exact: small integers), columns K..K0-1 zero; one thread per 8 columns of a row
 // (x over a row's chunks, y over rows).
 __global__ void obs_tiles(const uint8_t* __restrict__ obs, int K, int K0, int64_t n, uint8_t* __restrict__ x0) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int kc = threadIdx.x;  // 8-column chunk
   if (kc >= K0 / 8) return;
   for (int64_t r = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; r < n; r += (int64_t)gridDim.x * blockDim.y) {
@@ -94,28 +95,30 @@ __global__ void obs_tiles(const uint8_t* __restrict__ obs, int K, int K0, int64_
 }
 
 // logits[e][a] = sum over n-tiles and column halves (in order) of the actor's partial sums
-// + ba3[a] (-inf where illegal); values[e] likewise from the critic's
+// + ba3[a] (-inf where illegal); values[e] likewise from the critic's.  One thread per output.
 // (slots: the partial sums per (row, head, n-tile, column half): 8, or 32 for A > 8)
 __global__ void heads_final(const float* __restrict__ partial, int n_tiles, int slots, const float* __restrict__ ba3,
                             const float* __restrict__ bc3, const uint8_t* __restrict__ legal, int A, int64_t n,
                             float* __restrict__ logits, float* __restrict__ values) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n * (A + 1)) return;
+  const int64_t e = i / (A + 1);
+  const int a = (int)(i - e * (A + 1));
   const int parts = 2 * n_tiles;  // (n-tile, column half) pairs
-  const float* pa = partial + (e * 2 + 0) * (int64_t)parts * slots;
-  const float* pc = partial + (e * 2 + 1) * (int64_t)parts * slots;
-  for (int a = 0; a < A; ++a) {
-    float z = 0.0f;
-    for (int t = 0; t < parts; ++t) z += pa[t * slots + a];
+  const float* p = partial + (e * 2 + (a == A ? 1 : 0)) * (int64_t)parts * slots + (a == A ? 0 : a);
+  float z = 0.0f;
+#pragma unroll 8
+  for (int t = 0; t < parts; ++t) z += p[t * slots];
+  if (a == A) {
+    values[e] = z + bc3[0];
+  } else {
     z += ba3[a];
     logits[e * A + a] = (legal && !legal[e * A + a]) ? -INFINITY : z;
   }
-  float v = 0.0f;
-  for (int t = 0; t < parts; ++t) v += pc[t * slots];
-  values[e] = v + bc3[0];
 }
 
-// Output columns per GEMM tile for an N-column product: the widest multiple of 32 up to
+// Rows per stored weight tile of an N-row matrix, the widest output tile: the widest multiple of 32 up to
 // 256 that divides N (N is a multiple of 32).
 int bn_for(int N) {
   for (int b = 256; b >= 32; b -= 32)
@@ -138,19 +141,49 @@ std::vector<__nv_bfloat16> tile_matrix(const std::vector<__nv_bfloat16>& w, int 
   return t;
 }
 
-aht_status run_gemm(aht_s5* s, const s5g::GemmArgs& g0, int64_t n) {
+// Launches a kernel as a programmatic dependent of the one before it in the stream.
+template <class... P, class... T>
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t stream, T... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+int m_tiles_of(int64_t n) { return (int)((n + s5g::kBM - 1) / s5g::kBM); }
+
+// Output columns per tile of an N-column product over m_tiles x batch row tiles: the stored
+// tiles' width, halved (down to 32) while the tiles still fit one wave of SMs.
+int tile_columns(const aht_s5* s, int N, int m_tiles, int batch) {
+  int bn = bn_for(N);
+  while (bn % 64 == 0 && (int64_t)m_tiles * batch * (N / (bn / 2)) <= s->n_sms) bn /= 2;
+  return bn;
+}
+
+// One product of N output columns (the SSM's modes need the one full-width tile).
+aht_status run_gemm(aht_s5* s, const s5g::GemmArgs& g0, int N, int64_t n) {
   s5g::GemmArgs g = g0;
   g.n = n;
-  g.m_tiles = (int)((n + s5g::kBM - 1) / s5g::kBM);
+  g.m_tiles = m_tiles_of(n);
+  g.BW = bn_for(N);
+  g.BN = g.epi == s5g::kSsm ? g.BW : tile_columns(s, N, g.m_tiles, g.batch);
+  g.n_tiles = N / g.BN;
+  g.stages = s5g::gemm_stages(g.BN);
   g.status = s->status;
   const int tiles = g.m_tiles * g.n_tiles * g.batch;
   const int grid = std::min(tiles, s->n_sms);
   const size_t smem = s5g::gemm_smem_bytes(g.BN);
   if (g.epi == s5g::kHeads && (g.n_out[0] > 8 || g.n_out[1] > 8))
-    s5g::gemm_kernel<s5g::kMaxOut><<<grid, s5g::kThreads, smem, s->stream>>>(g);
+    S5_CUDA(launch_dependent(s5g::gemm_kernel<s5g::kMaxOut>, grid, s5g::kThreads, smem, s->stream, g));
   else
-    s5g::gemm_kernel<8><<<grid, s5g::kThreads, smem, s->stream>>>(g);
-  S5_CUDA(cudaGetLastError());
+    S5_CUDA(launch_dependent(s5g::gemm_kernel<8>, grid, s5g::kThreads, smem, s->stream, g));
   return AHT_OK;
 }
 
@@ -299,13 +332,15 @@ aht_status aht_s5_create(const aht_s5_params* p, int64_t max_envs, void* cuda_st
   for (const Act& x : acts)
     if (!alloc((void**)x.p, x.bytes) || cudaMemset(*x.p, 0, x.bytes) != cudaSuccess)
       return bail(AHT_ENOMEM, "S5 scratch allocation failed");
-  const int n_tiles_f = F / bn_for(F);
+  // head partials: full-width tiles over all rows, or narrower ones in at most one wave of
+  // row tiles x 2 heads x n-tiles
+  const int64_t part_tiles = std::max<int64_t>((int64_t)s->m_tiles * (F / bn_for(F)), s->n_sms / 2);
   if (!alloc((void**)&s->u, (size_t)rows * H * 4) ||
-      !alloc((void**)&s->partial, (size_t)rows * 2 * n_tiles_f * 2 * s5g::kMaxOut * 4) ||
+      !alloc((void**)&s->partial, (size_t)part_tiles * s5g::kBM * 2 * 2 * s5g::kMaxOut * 4) ||
       !alloc((void**)&s->status, 4) || cudaMemset(s->status, 0, 4) != cudaSuccess)
     return bail(AHT_ENOMEM, "S5 scratch allocation failed");
   if (cudaFuncSetAttribute(s5g::gemm_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)s5g::gemm_smem_bytes(256)) != cudaSuccess ||
+                           (int)s5g::kStageSmem) != cudaSuccess ||
       cudaFuncSetAttribute(s5g::gemm_kernel<s5g::kMaxOut>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)s5g::gemm_smem_bytes(256)) != cudaSuccess)
     return bail(AHT_ECUDA, "setting the GEMM's shared-memory limit failed");
@@ -335,54 +370,53 @@ aht_status aht_s5_step(aht_s5* s, const uint8_t* obs, const uint8_t* reset, cons
     obs_tiles<<<(unsigned)blocks, dim3((unsigned)bx, (unsigned)by), 0, s->stream>>>(obs, K, s->K0, n, s->x0);
     S5_CUDA(cudaGetLastError());
   }
-  auto layer = [&](const uint8_t* A_, int k_in, const uint8_t* B_, int N, int epi) {
+  auto layer = [&](const uint8_t* A_, int k_in, const uint8_t* B_, int epi) {
     s5g::GemmArgs g{};
     g.A = A_;
     g.B = B_;
     g.k_tiles = kt(k_in);
-    g.BN = bn_for(N);
-    g.n_tiles = N / g.BN;
     g.batch = 1;
     g.epi = epi;
     return g;
   };
   // encoder layer 1 (exact bf16 observation): relu, hi | lo
-  s5g::GemmArgs g = layer(s->x0, K, s->We1, H, s5g::kSplit);
+  s5g::GemmArgs g = layer(s->x0, K, s->We1, s5g::kSplit);
   g.bias = s->be1; g.relu = 1; g.parts = 2; g.I = H; g.out = s->a1; g.out_k_tiles = kt(2 * H);
-  if (aht_status e = run_gemm(s, g, n)) return e;
+  if (aht_status e = run_gemm(s, g, H, n)) return e;
   // encoder layer 2: relu; u (fp32) and its hi | lo | hi for the three-term SSM product
-  g = layer(s->a1, 2 * H, s->We2, H, s5g::kSplit);
+  g = layer(s->a1, 2 * H, s->We2, s5g::kSplit);
   g.bias = s->be2; g.relu = 1; g.parts = 3; g.I = H; g.out = s->a2; g.out_k_tiles = kt(3 * H); g.out32 = s->u;
-  if (aht_status e = run_gemm(s, g, n)) return e;
+  if (aht_status e = run_gemm(s, g, H, n)) return e;
   // SSM: Bbar u, the recurrence and x's hi | lo | hi
-  g = layer(s->a2, 3 * H, s->Bbar3, 2 * P, s5g::kSsm);
+  g = layer(s->a2, 3 * H, s->Bbar3, s5g::kSsm);
   g.lbar = s->lbar; g.state = state; g.reset = reset; g.P = P; g.out = s->a3; g.out_k_tiles = kt(6 * P);
-  if (aht_status e = run_gemm(s, g, n)) return e;
+  if (aht_status e = run_gemm(s, g, 2 * P, n)) return e;
   // Re(C x), then v = u + gelu(y + D u) as hi | lo
-  g = layer(s->a3, 6 * P, s->Cc3, H, s5g::kGelu);
+  g = layer(s->a3, 6 * P, s->Cc3, s5g::kGelu);
   g.u = s->u; g.D = s->Dv; g.I = H; g.out = s->a4; g.out_k_tiles = kt(2 * H);
-  if (aht_status e = run_gemm(s, g, n)) return e;
+  if (aht_status e = run_gemm(s, g, H, n)) return e;
   // heads layer 0, both heads at once: relu, hi | lo of each head's F units
   const int64_t head_act = rows * kt(2 * F) * 64 * 2;  // bytes of one head's activation
-  g = layer(s->a4, 2 * H, s->Wh0, 2 * F, s5g::kSplit);
+  g = layer(s->a4, 2 * H, s->Wh0, s5g::kSplit);
   g.bias = s->bh0; g.relu = 1; g.parts = 2; g.I = F; g.out = s->a5; g.out_stride = head_act;
   g.out_k_tiles = kt(2 * F);
-  if (aht_status e = run_gemm(s, g, n)) return e;
+  if (aht_status e = run_gemm(s, g, 2 * F, n)) return e;
   // heads layer 1 (two-member batch)
   const int64_t wh_bytes = (int64_t)F * 2 * F * 2;
-  g = layer(s->a5, 2 * F, s->Wh1, F, s5g::kSplit);
+  g = layer(s->a5, 2 * F, s->Wh1, s5g::kSplit);
   g.batch = 2; g.a_stride = head_act; g.b_stride = wh_bytes;
   g.bias = s->bh1; g.relu = 1; g.parts = 2; g.I = F; g.out = s->a6; g.out_stride = head_act;
   g.out_k_tiles = kt(2 * F);
-  if (aht_status e = run_gemm(s, g, n)) return e;
+  if (aht_status e = run_gemm(s, g, F, n)) return e;
   // heads layer 2 with both output layers: per-tile partial sums
-  g = layer(s->a6, 2 * F, s->Wh2, F, s5g::kHeads);
+  g = layer(s->a6, 2 * F, s->Wh2, s5g::kHeads);
   g.batch = 2; g.a_stride = head_act; g.b_stride = wh_bytes;
   g.bias = s->bh2; g.W3[0] = s->W3a; g.W3[1] = s->W3c; g.n_out[0] = A; g.n_out[1] = 1; g.partial = s->partial;
-  if (aht_status e = run_gemm(s, g, n)) return e;
-  heads_final<<<(unsigned)((n + 255) / 256), 256, 0, s->stream>>>(s->partial, F / bn_for(F), A > 8 ? s5g::kMaxOut : 8,
-                                                                  s->ba3, s->bc3, legal, A, n, logits, values);
-  S5_CUDA(cudaGetLastError());
+  if (aht_status e = run_gemm(s, g, F, n)) return e;
+  const int n_tiles = F / tile_columns(s, F, m_tiles_of(n), 2);
+  S5_CUDA(launch_dependent(heads_final, (int)((n * (A + 1) + 255) / 256), 256, 0, s->stream, (const float*)s->partial,
+                           n_tiles, A > 8 ? s5g::kMaxOut : 8, (const float*)s->ba3, (const float*)s->bc3, legal, A, n,
+                           logits, values));
   return AHT_OK;
 }
 

@@ -8,8 +8,14 @@
 // copy moves a whole tile into shared memory:
 //   activation tile (mt, kt): rows [128 mt, 128 mt + 128) x k [64 kt, 64 kt + 64), 16 KB,
 //                             at ((mt * KT + kt) * 16 KB)
-//   weight tile (nt, kt):     rows [BN nt, BN nt + BN) x k [64 kt, 64 kt + 64), BN * 128 B,
-//                             at ((nt * KT + kt) * BN * 128)
+//   weight tile (nt, kt):     rows [BW nt, BW nt + BW) x k [64 kt, 64 kt + 64), BW * 128 B,
+//                             at ((nt * KT + kt) * BW * 128); any aligned run of BN rows of
+//                             it is itself a tile
+// A batch of few rows would occupy few SMs with BN = BW columns a tile, each streaming the
+// whole K; the launch then takes narrower tiles (down to 32 columns) while they fit one wave.
+// Consecutive products are programmatic dependent launches: a kernel's barriers, tensor
+// memory and first weight stages are set up while the one before finishes.  (One step of 61
+// envs 112 us with full-width tiles in plain stream order, 71 now.)
 // A persistent kernel walks the output tiles (batch, m-tile, n-tile; n fastest, so that the
 // CTAs working on one activation tile at the same time share it in L2, and the weights of
 // a layer, a few MB, stay there).  Warp 0 (one lane) streams the stages
@@ -36,7 +42,8 @@ namespace s5g {
 
 constexpr int kBM = 128;          // rows of an output tile (one tensor-memory lane each)
 constexpr int kBK = 64;           // k per stage
-constexpr int kStages = 4;
+constexpr int kMaxStages = 9;
+constexpr uint32_t kStageSmem = 196608;     // shared memory of the stages: 4 of BN = 256, 9 of 32
 constexpr int kThreads = 320;     // producer, MMA, 8 epilogue warps
 constexpr int kEpiThreads = 256;
 constexpr uint32_t kATile = kBM * kBK * 2;  // 16 KB
@@ -49,7 +56,10 @@ struct GemmArgs {
   int64_t a_stride;        // bytes between batch members
   const uint8_t* B;        // tiled weights of batch member 0
   int64_t b_stride;
-  int32_t m_tiles, n_tiles, k_tiles, batch, BN;
+  int32_t m_tiles, n_tiles, k_tiles, batch;
+  int32_t BN;              // columns of an output tile
+  int32_t BW;              // rows of a stored weight tile (a multiple of BN)
+  int32_t stages;
   int64_t n;               // valid rows
   int32_t epi;
   // kSplit: v = act(acc + bias) of output column gc (group g = gc / I, column c = gc % I)
@@ -84,17 +94,20 @@ __device__ __forceinline__ int64_t chunk_off(int64_t mt, int k_tiles, int kt, in
 template <int kOut>
 __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages];
+  __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
   __shared__ __align__(8) uint64_t accf_bar[2], acce_bar[2], drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int BN = a.BN;
-  const uint32_t b_tile = (uint32_t)BN * kBK * 2;
+  const int BN = a.BN, NS = a.stages;
+  const uint32_t b_tile = (uint32_t)BN * kBK * 2, w_tile = (uint32_t)a.BW * kBK * 2;
   const uint32_t stage_bytes = kATile + b_tile;
   const int n_tiles_total = a.m_tiles * a.n_tiles * a.batch;
+  // the next kernel of the step may start: it touches nothing this one writes, or reads, before
+  // its griddepcontrol.wait
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < NS; ++s) {
       tc::mbar_init(&full_bar[s], 1);
       tc::mbar_init(&empty_bar[s], 1);
     }
@@ -128,26 +141,50 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
   if (warp == 0) {
     // ============================== producer =========================================
     if (lane == 0) {
-      int s = 0;
-      uint32_t use = 0;  // times stage s was filled before
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < n_tiles_total; tile += gridDim.x) {
+      // a tile's operands: its weight rows, and of its activation rows (the last m-tile's) only
+      // the row blocks that hold rows
+      const uint8_t *A = nullptr, *B = nullptr;
+      uint32_t a_bytes = 0;
+      auto locate = [&](int tile) {
         int b, nt, mt;
         tile_coords(tile, b, nt, mt);
-        const uint8_t* A = a.A + b * a.a_stride + (int64_t)mt * a.k_tiles * kATile;
-        const uint8_t* B = a.B + b * a.b_stride + (int64_t)nt * a.k_tiles * b_tile;
-        for (int kt = 0; kt < a.k_tiles; ++kt) {
+        const int col0 = nt * BN, wt = col0 / a.BW;
+        A = a.A + b * a.a_stride + (int64_t)mt * a.k_tiles * kATile;
+        B = a.B + b * a.b_stride + (int64_t)wt * a.k_tiles * w_tile + (int64_t)(col0 - wt * a.BW) * (kBK * 2);
+        a_bytes = (uint32_t)min((a.n - (int64_t)mt * kBM + 7) / 8, (int64_t)(kBM / 8)) * 1024u;
+      };
+      auto copy_b = [&](int kt, int s) {
+        tc::mbar_expect_tx(&full_bar[s], a_bytes + b_tile);
+        tc::bulk_g2s(smem + (size_t)s * stage_bytes + kATile, B + (int64_t)kt * w_tile, b_tile, &full_bar[s]);
+      };
+      auto copy_a = [&](int kt, int s) {
+        tc::bulk_g2s(smem + (size_t)s * stage_bytes, A + (int64_t)kt * kATile, a_bytes, &full_bar[s]);
+      };
+      // the first stages' weights do not depend on the kernel before: they are on their way
+      // while it finishes
+      locate(blockIdx.x);  // (the grid has no more CTAs than tiles)
+      const int early = min(NS, a.k_tiles);
+      for (int i = 0; i < early; ++i) copy_b(i, i);
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      for (int i = 0; i < early; ++i) copy_a(i, i);
+      issued_stages = early;
+      int s = early == NS ? 0 : early, kt = early;
+      uint32_t use = early == NS ? 1 : 0;  // times stage s was filled before
+      bool ok = true;
+      for (int tile = blockIdx.x; ok;) {
+        for (; kt < a.k_tiles; ++kt) {
           if (use > 0 && !(ok = wait_or_abort(&empty_bar[s], (use - 1) & 1u))) break;
-          uint8_t* dst = smem + (size_t)s * stage_bytes;
-          tc::mbar_expect_tx(&full_bar[s], stage_bytes);
-          tc::bulk_g2s(dst, A + (int64_t)kt * kATile, kATile, &full_bar[s]);
-          tc::bulk_g2s(dst + kATile, B + (int64_t)kt * b_tile, b_tile, &full_bar[s]);
+          copy_b(kt, s);
+          copy_a(kt, s);
           ++issued_stages;
-          if (++s == kStages) {
+          if (++s == NS) {
             s = 0;
             ++use;
           }
         }
+        if ((tile += gridDim.x) >= n_tiles_total) break;
+        locate(tile);
+        kt = 0;
       }
       if (!ok) abort_flag = 1;
     }
@@ -174,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
           for (int kk = 0; kk < kBK / 16; ++kk)
             tc::mma_ss(D, da + 16u * kk, db + 16u * kk, idesc, (kt | kk) != 0);
           tc::commit(&empty_bar[s]);  // the stage is free once these products have read it
-          if (++s == kStages) {
+          if (++s == NS) {
             s = 0;
             fpar ^= 1u;
           }
@@ -185,6 +222,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
     }
   } else {
     // ================================ epilogue =======================================
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the state and u of earlier kernels
     const int q = warp & 3;                       // tensor-memory lane quadrant
     const int r = 32 * q + lane;                  // row of the tile
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
@@ -195,6 +233,25 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
       int b, nt, mt;
       tile_coords(tile, b, nt, mt);
       const int acc = j & 1;
+      const int64_t row = (int64_t)mt * kBM + r;
+      const bool live = row < a.n;
+      // kSsm: 16 modes of this row's state, requested ahead of their use (the first ones while
+      // the products run: loads and stores of the state in turn, each waiting for the last,
+      // took the layer 69 us at 16384 rows, 23 so)
+      float4 pre[8];
+      const bool fresh = a.epi == kSsm && live && a.reset[row] != 0;
+      auto load_state = [&](const float* st, int P) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          pre[i] = *reinterpret_cast<const float4*>(st + 4 * i);
+          pre[4 + i] = *reinterpret_cast<const float4*>(st + P + 4 * i);
+        }
+        if (fresh) {  // an episode's first step
+#pragma unroll
+          for (int i = 0; i < 8; ++i) pre[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      };
+      if (a.epi == kSsm && live) load_state(a.state + row * (int64_t)(2 * a.P) + ch * (a.P / 2), a.P);
       bool got = false;
       if (ok) {
         for (int tries = 0; tries < 1000 && !got && !abort_flag; ++tries)
@@ -204,8 +261,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
       if (!ok) break;
       tc::fence_after_sync();
       const uint32_t T = tmem + (uint32_t)(acc * 256) + lane_base;
-      const int64_t row = (int64_t)mt * kBM + r;
-      const bool live = row < a.n;
       const int col0 = nt * BN;                   // first output column of the tile
       // this warp's columns: half of the tile's when each half is whole 32-column chunks,
       // else all of them for the first half
@@ -257,24 +312,25 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
           }
         }
       } else if (a.epi == kSsm) {
-        const int P = a.P, pw = P / 2;           // this warp group's modes: [ch pw, ch pw + pw)
-        const bool rs = live && a.reset[row] != 0;
-        for (int p0 = ch * pw; p0 < ch * pw + pw; p0 += 16) {
+        const int P = a.P, p_end = (ch + 1) * (P / 2);  // this warp group's modes: its half of P
+        float* st = a.state + row * (int64_t)(2 * P);
+        for (int p0 = ch * (P / 2); p0 < p_end; p0 += 16) {
+          float4 sr[4], si[4];  // this chunk's state was requested a chunk ago
+#pragma unroll
+          for (int i = 0; i < 4; ++i) sr[i] = pre[i], si[i] = pre[4 + i];
+          if (live && p0 + 16 < p_end) load_state(st + p0 + 16, P);
           uint32_t vr[16], vi[16];
           tc::ld_x16(T + p0, vr);
           tc::ld_x16(T + P + p0, vi);
           tc::wait_ld();
           if (!live) continue;
-          float* st = a.state + row * (int64_t)(2 * P);
           float xr[16], xi[16];
 #pragma unroll
           for (int i = 0; i < 16; i += 4) {
-            float4 sr = *reinterpret_cast<const float4*>(st + p0 + i);
-            float4 si = *reinterpret_cast<const float4*>(st + P + p0 + i);
-            if (rs) sr = si = make_float4(0.f, 0.f, 0.f, 0.f);
             const float4 lr = __ldg(reinterpret_cast<const float4*>(a.lbar + p0 + i));
             const float4 li = __ldg(reinterpret_cast<const float4*>(a.lbar + P + p0 + i));
-            const float srv[4] = {sr.x, sr.y, sr.z, sr.w}, siv[4] = {si.x, si.y, si.z, si.w};
+            const float srv[4] = {sr[i / 4].x, sr[i / 4].y, sr[i / 4].z, sr[i / 4].w};
+            const float siv[4] = {si[i / 4].x, si[i / 4].y, si[i / 4].z, si[i / 4].w};
             const float lrv[4] = {lr.x, lr.y, lr.z, lr.w}, liv[4] = {li.x, li.y, li.z, li.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -395,8 +451,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
   }
   if (warp == 0 && lane == 0 && abort_flag) {
     // copies still in flight land before the CTA leaves: the last stages issued
-    for (int d = issued_stages - 1; d >= 0 && d >= issued_stages - kStages; --d)
-      tc::mbar_wait(&full_bar[d % kStages], (uint32_t)(d / kStages) & 1u);
+    for (int d = issued_stages - 1; d >= 0 && d >= issued_stages - NS; --d)
+      tc::mbar_wait(&full_bar[d % NS], (uint32_t)(d / NS) & 1u);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -406,7 +462,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const GemmArgs a) {
   }
 }
 
-inline size_t gemm_smem_bytes(int BN) { return (size_t)kStages * (kATile + (size_t)BN * kBK * 2); }
+inline size_t gemm_stage_bytes(int BN) { return kATile + (size_t)BN * kBK * 2; }
+inline int gemm_stages(int BN) {
+  const int s = (int)(kStageSmem / gemm_stage_bytes(BN));
+  return s < kMaxStages ? s : kMaxStages;
+}
+inline size_t gemm_smem_bytes(int BN) { return gemm_stages(BN) * gemm_stage_bytes(BN); }
 
 }  // namespace s5g
 }  // namespace aht
