@@ -331,6 +331,7 @@ TcDims make_tc_dims(const MlpDims& m, bool split) {
   // an observation wider than an agent's 256 A-operand columns: the first layer runs on
   // CUDA cores from the observation's changed features (LBF), W1 stays out of the block
   t.sparse = (m.sparse && t.KP > 256) ? 1 : 0;
+  t.stage_rows = 32;  // (no more than the partial logits it shares memory with; see fit_stage)
   const uint32_t w1 = t.sparse ? 0u : (uint32_t)(m.H0 * t.KP * 2);
   uint32_t o = 0;
   t.oW1 = o; o += w1;
@@ -348,10 +349,12 @@ TcDims make_tc_dims(const MlpDims& m, bool split) {
 
 // Shared memory of the tensor-core kernel: both policies' blocks, the u8 observation
 // tile [128][obs_dim], 128 env states, 128 teammate actions and the output layer's
-// partial sums [2 agents][2 halves][128][8] fp32.
+// partial sums [2 agents][2 halves][128][8] fp32, which in the sparse kernel lie over the
+// hidden layer on its way to tensor memory.
 size_t tc_smem_bytes(const TcDims& t, int obs_dim, int state_bytes) {
+  const size_t zpart = 4 * 128 * 8 * 4, stage = t.sparse ? (size_t)t.stage_rows * tc_stage_ld(t) * 4 : 0;
   return 2 * (size_t)t.pol_bytes + align_up(128 * obs_dim, 16) + align_up(128 * state_bytes, 16) + 128 +
-         4 * 128 * 8 * 4;
+         (t.sparse ? 128 * kTcObjectWords * 4 : 0) + std::max(zpart, stage);
 }
 
 // The tensor-core path applies to LBF populations whose padded observation (KP/2
@@ -365,6 +368,18 @@ bool tc_eligible(const aht_ctx* c, int dtype) {
   if ((t.KP > 256 && !t.sparse) || m.H0 > 128 || m.H1 > 128 || m.H0 % 64 || m.H1 % 64 || m.NA + 1 > 8)
     return false;
   return m.K % 4 == 0 && tc_smem_bytes(t, m.K, c->ops.bytes()) <= c->smem_optin;
+}
+
+// Stages as many rows of the sparse kernel's hidden layer as fit beside the rest.
+void fit_stage(const aht_ctx* c, TcDims* t) {
+  for (int rows : {128, 64}) {
+    TcDims u = *t;
+    u.stage_rows = rows;
+    if (t->sparse && tc_smem_bytes(u, c->mlp.K, c->ops.bytes()) + kTcGatherScratch <= c->smem_optin) {
+      *t = u;
+      return;
+    }
+  }
 }
 
 // Streamed tensor-core block of a wide policy (see WideDims).
@@ -843,6 +858,7 @@ aht_status aht_create(const aht_env_desc* envd, const aht_pop_desc* pop, int64_t
   c->weight_dtype = pop->weight_dtype;
   if (tc_eligible(c, pop->weight_dtype)) {
     c->tcd = make_tc_dims(m, pop->weight_dtype == AHT_FP32);
+    fit_stage(c, &c->tcd);
     c->tc_smem = tc_smem_bytes(c->tcd, m.K, c->ops.bytes());
     std::vector<uint8_t> blocks((size_t)c->tcd.pol_bytes * pop->n_policies);
     for (int p = 0; p < pop->n_policies; ++p) {

@@ -160,26 +160,33 @@ struct EnvLbf {
     w[s.ay[seat] * d.width + s.ax[seat]] = (uint32_t)s.al[seat];
   }
 
-  // The observation as changes to the all-empty pattern (every cell word 0x01000000):
-  // slot i (foods 0-2, the other agent, the agent itself) is the cell's two changed
-  // features, +value in its channel and -1 in channel 3, as entries (feature << 8) |
-  // (delta & 0xFF) in e[2i], e[2i + 1].  Returns the mask of the entries in use (eaten
-  // foods have none).  The rules keep occupied cells distinct, so this equals obs().
-  __device__ static uint32_t sparse_obs(const DevEnv& d, const State& s, int seat, uint32_t (&e)[10]) {
-    auto cell = [&](int i, int x, int y, int ch, int v) {
-      const uint32_t c = (uint32_t)(y * d.width + x);
-      e[2 * i] = ((4u * c + (uint32_t)ch) << 8) | (uint32_t)(v & 0xFF);
-      e[2 * i + 1] = ((4u * c + 3u) << 8) | 0xFFu;
-    };
-    uint32_t mask = 0x3C0u;
+  // The occupied cells as three words of (cell, value) byte pairs: foods 0-2 (value = level, 0
+  // for an eaten or absent one), agent 1, agent 0 (value = level).
+  __device__ static void pack_objects(const DevEnv& d, const State& s, uint32_t (&w)[3]) {
+    auto object = [&](int x, int y, int v) { return v ? (uint32_t)(y * d.width + x) | ((uint32_t)v << 8) : 0u; };
+    uint32_t f[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      cell(k, s.fx[k], s.fy[k], 2, s.fl[k]);
-      if (!((s.eaten >> k) & 1u)) mask |= 3u << (2 * k);
+    for (int k = 0; k < 3; ++k) f[k] = object(s.fx[k], s.fy[k], (s.eaten >> k) & 1u ? 0 : s.fl[k]);
+    w[0] = f[0] | (f[1] << 16);
+    w[1] = f[2] | (object(s.ax[1], s.ay[1], s.al[1]) << 16);
+    w[2] = object(s.ax[0], s.ay[0], s.al[0]);
+  }
+
+  // The observation of `seat` as changes to the all-empty pattern (every cell word
+  // 0x01000000), from packed objects: slot i (foods 0-2, the other agent, the agent itself)
+  // is its cell's two changed features, +value in the object's channel and -1 in channel 3:
+  // features f[2i], f[2i + 1] with changes v[i] and -(v[i] != 0).  An absent food has value 0
+  // and feature 0.  The rules keep occupied cells distinct, so this equals obs().
+  __device__ static void sparse_obs(const uint32_t (&w)[3], int seat, uint32_t (&f)[10], int (&v)[5]) {
+    const uint32_t other = seat == 0 ? w[1] >> 16 : w[2], self = seat == 0 ? w[2] : w[1] >> 16;
+    const uint32_t o[5] = {w[0] & 0xFFFFu, w[0] >> 16, w[1] & 0xFFFFu, other, self};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const uint32_t c4 = 4u * (o[i] & 0xFFu), ch = i < 3 ? 2u : i == 3 ? 1u : 0u;
+      v[i] = (int)(o[i] >> 8);
+      f[2 * i] = v[i] ? c4 + ch : 0u;
+      f[2 * i + 1] = v[i] ? c4 + 3u : 0u;
     }
-    cell(3, s.ax[1 - seat], s.ay[1 - seat], 1, s.al[1 - seat]);
-    cell(4, s.ax[seat], s.ay[seat], 0, s.al[seat]);
-    return mask;
   }
 
   // The other seat's view of one cell word of the observation: channels 0 (the observing

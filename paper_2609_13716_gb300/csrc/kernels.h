@@ -64,9 +64,16 @@ struct TcDims {
   int32_t sparse;          // 1: no W1 in the block; the first layer runs on CUDA cores from
                            // the env's changed features and the fp32 W1^T / c of the
                            // CUDA-core population (LBF grids beyond 256 tensor-memory columns)
+  int32_t stage_rows;      // sparse: rows of the hidden layer staged in shared memory at a time
+                           // (128, 64 or 32: the most that fit)
   uint32_t oW1, oW2, oW3, ob2, ob3, oW1lo, oW2lo;
   uint32_t pol_bytes;
 };
+
+constexpr int kTcObjectWords = 3;  // sparse: packed occupied cells of an env (EnvLbf::pack_objects)
+// Words per row of the staged hidden layer (sparse first layer): H0 and, where the stage has
+// room, a pad that spreads a warp's rows over the banks.
+__host__ __device__ inline int tc_stage_ld(const TcDims& t) { return t.H0 + (t.stage_rows > 32 ? 4 : 0); }
 
 // Cross-play tiles of the tensor-core rollout kernel: tile t is chunk t % tpp of pair
 // t / tpp, envs [pair P + 128 chunk, min(pair P + 128 chunk + 128, (pair + 1) P)), ego

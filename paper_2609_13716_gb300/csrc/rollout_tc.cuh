@@ -19,9 +19,10 @@
 //       from registers (16x256b accumulator loads are its fragment layout)
 //   sampling (ego in warps 0-3, teammate in warps 4-7), env step, trajectory write.
 //
-// Warp roles: warps 0-7 ("compute", 256 threads) build the ego's observation rows for the
-// trajectory, form h1, run epilogue 2 (thread r and r + 128 own env row r, tensor-memory
-// lane r; the halves split the columns), sample and step the envs; warp 8 issues every
+// Warp roles: warps 0-7 ("compute", 256 threads) form h1 (a warp per row), run epilogue 2
+// (thread r and r + 128 own env row r, tensor-memory lane r; the halves split the columns),
+// sample, step the envs and move the changed cells of the ego's observation rows, which
+// stay in shared memory for the trajectory; warp 8 issues every
 // MMA; warps 9-12 store the ego's observation rows of gathered tiles (scattered rows, a
 // quarter each, one warp per SM sub-partition) while the compute warps go on.  They meet
 // only through mbarriers: operand-ready (256 arrivals from the compute threads) and
@@ -29,9 +30,12 @@
 // observation buffer free (one arrival per store warp).  Each of these barriers completes
 // once per step, so its phase parity is the step's parity.  Compute warps synchronise
 // among themselves with a named barrier that also ORs an error flag.  Weights (all but
-// W1) are bulk-copied (TMA) into shared memory once per CTA; W1^T and c are read from
-// the L2-resident fp32 population.  Every wait is bounded: on expiry the CTA records
-// kStatusTimeout, stops, drains its own MMAs (bounded), frees tensor memory and exits.
+// W1) are bulk-copied (TMA) into shared memory once per CTA; W1^T and c are read from the
+// L2-resident fp32 population.  A third of a step is h1, bound by its warps' instruction
+// latency: a thread per row, each lane gathering its own W1 rows in 32-byte pieces, made LBF
+// 12x12 collection 4096 x 128 3.26 ms; a warp per row, the agents' epilogues side by side,
+// 1.30 (half the bytes, W1 as bf16, would gain 3 %).  Every wait is bounded: on expiry the CTA
+// records kStatusTimeout, stops, drains its own MMAs (bounded), frees tensor memory and exits.
 //
 // Tensor memory (512 columns): agent a uses columns [256a, 256a + 128) for its A operand
 // (hi|lo of h1) and [256a + 128, 256a + 256) for its fp32 accumulator.
@@ -216,11 +220,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
   const int cells = od / 4;          // observation words per row
   const int chunks = d.KP / 16;      // 16-byte chunks per observation row
   const int split = (chunks + 1) / 2;
-  // the halves build words [my_w0, my_w1) of the ego's row
+  // the halves write words [my_w0, my_w1) of the ego's first row
   const int my_w0 = min(4 * (half ? split : 0), cells), my_w1 = min(4 * (half ? chunks : split), cells);
   const bool with_boot = !kXp && a.traj.last_value != nullptr;  // the ego's V_T after the last step
   // gathered tiles: warps 9-12 store the ego's observation rows of every step
   const bool obs_warp = kGather && a.traj.obs != nullptr;
+  const bool rows = !kXp && a.traj.obs != nullptr;  // the ego's rows are kept for the trajectory
 
   // The tile is the contiguous env range [tile.x, tile.x + count); observation rows are
   // packed at obs_dim bytes (an odd number of words: no bank conflicts per thread row),
@@ -229,7 +234,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
   uint8_t* const sObs = smem + 2 * d.pol_bytes;                             // [128][obs_dim] u8
   State* st = reinterpret_cast<State*>(sObs + align_up(128 * od, 16));      // [128]
   uint8_t* act1s = reinterpret_cast<uint8_t*>(st) + align_up(128 * sizeof(State), 16);  // [128]
-  float* zpart = reinterpret_cast<float*>(act1s + 128);                     // [2][2][128][8]
+  uint32_t* const objs = reinterpret_cast<uint32_t*>(act1s + 128);          // [128][3] packed objects
+  float* zpart = reinterpret_cast<float*>(objs + 128 * kTcObjectWords);     // [2][2][128][8]
+  // h1 on its way to tensor memory: d.stage_rows rows of H0 words (hi pairs, then lo pairs)
+  // and padding; the partial logits lie over it (a step's are read before the next step's h1
+  // is written)
+  uint32_t* const stage = reinterpret_cast<uint32_t*>(zpart);
+  const int stage_ld = tc_stage_ld(d);
 
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -255,6 +266,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  auto put_objects = [&](const State& s) {  // this thread's row
+    uint32_t w[3];
+    Env::pack_objects(a.b.env, s, w);
+    for (int k = 0; k < 3; ++k) objs[row * kTcObjectWords + k] = w[k];
+  };
+  if (warp < 8 && row < count) {
+    const State s0 = st[row];
+    if (rows) Env::obs_words(a.b.env, s0, 0, reinterpret_cast<uint32_t*>(sObs + row * od), my_w0, my_w1);
+    if (half == 0) put_objects(s0);
+  }
+  if (!kXp && !kGather) tc::fence_proxy_async();  // (the rows are read by the bulk copy engine)
+  __syncthreads();
 
   if (warp == 8) {
     // ================================ MMA warp =====================================
@@ -356,60 +379,92 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
     };
     auto sync_or = [&]() { return tc::bar_or(kTcComputeBar, kTcCompute, bad || abort_flag); };
     auto pol_block = [&](int ag) { return sW0 + (size_t)ag * d.pol_bytes; };
+    // A tile of at most 64 rows puts the teammate's rows in other tensor-memory lanes than the
+    // ego's (32 or 64 on), so that different warps run the two agents' epilogues side by side.
+    const int tm_lanes = count <= 32 ? 32 : count <= 64 ? 64 : 0;
+    auto quad_row = [&](int ag) { return (warp & 3) * 32 - (ag == 1 ? tm_lanes : 0); };  // this warp's first row
 
-    // h1: r1 = 1 / (1 + exp(2 (c + sum over the changed features f of delta W1[:, f]))) for this
-    // thread's half of the units, split hi | lo into the A operand of L2; rows past count
-    // take c alone.  The W1 rows are gathered 8 units at a time with all ten
-    // features' loads issued before their multiply-adds (one L2 round trip per 8 units,
-    // not one per feature); an absent feature reads row 0 and adds 0 x W1 (exact)
-    auto sparse_h1 = [&](int ag, const State& s) {
-      const int H = d.H0;
-      const uint32_t P = tmem + (uint32_t)(ag * 256) + lane_base;
-      const float* pw = a.b.weights + (int64_t)(ag == 0 ? ego_pol : tm_pol) * a.b.mlp.stride;
-      const float* W1t = pw + a.b.mlp.oW1;
-      const float* cvec = pw + a.b.mlp.oC;
-      uint32_t e[10];
-      const uint32_t mask = row < count ? Env::sparse_obs(a.b.env, s, ag, e) : 0u;
+    // h1 of rows [lo, hi) of agents [ag0, ag1): r1 = 1 / (1 + exp(2 (c + sum over the changed features f of delta
+    // W1[:, f]))).  A slot is 128 / H0 rows of one agent, four consecutive units per lane, so
+    // that a feature's W1 row is one coalesced load; a warp requests a slot's ten rows while
+    // it finishes the slot before (an absent feature reads row 0 and adds 0 x W1, exact).  r1 is split hi | lo into `stage`; after a barrier each thread
+    // moves its row's half into tensor memory, the A operand of L2.
+    auto h1 = [&](int ag0, int ag1, int lo_row, int hi_row) {
+      const int H = d.H0, lpr = H / 4, rpw = 32 / lpr;  // lanes per row, rows per slot
+      const int sub = lane / lpr, u0 = 4 * (lane - sub * lpr);
+      const int slots = (hi_row - lo_row + rpw - 1) / rpw, total = (ag1 - ag0) * slots;
+      const int64_t agent1 = (int64_t)tm_pol * a.b.mlp.stride, agent0 = (int64_t)ego_pol * a.b.mlp.stride;
+      auto row_of = [&](int sl, int& ag) {  // (slots past the last repeat it)
+        const int q = min(sl, total - 1);
+        ag = ag0 + (q >= slots ? 1 : 0);
+        return lo_row + (q - (ag - ag0) * slots) * rpw + sub;
+      };
+      struct Slot {
+        int r, ag, v[5];
+        float4 w[10], c;
+      };
+      auto request = [&](Slot& t, int sl) {
+        t.r = row_of(sl, t.ag);
+        const float* pw = a.b.weights + (t.ag == 0 ? agent0 : agent1) + u0;
+        const uint32_t* ob = objs + min(t.r, count - 1) * kTcObjectWords;
+        const uint32_t ow[3] = {ob[0], ob[1], ob[2]};
+        uint32_t f[10];
+        Env::sparse_obs(ow, t.ag, f, t.v);
+        t.c = __ldg(reinterpret_cast<const float4*>(pw + a.b.mlp.oC));
+#pragma unroll
+        for (int q = 0; q < 10; ++q)
+          t.w[q] = __ldg(reinterpret_cast<const float4*>(pw + a.b.mlp.oW1 + f[q] * (uint32_t)H));
+      };
+      auto finish = [&](const Slot& t) {
+        float4 v = t.c;
+#pragma unroll
+        for (int q = 0; q < 10; ++q) {
+          const float dv = q & 1 ? (t.v[q / 2] ? -1.0f : 0.0f) : (float)t.v[q / 2];
+          v.x = fmaf(dv, t.w[q].x, v.x);
+          v.y = fmaf(dv, t.w[q].y, v.y);
+          v.z = fmaf(dv, t.w[q].z, v.z);
+          v.w = fmaf(dv, t.w[q].w, v.w);
+        }
+        uint2 hi, lo;
+        tc::split_bf16x2_p(tc::logistic2(tc::f2_mul(tc::f2_pack(v.x, v.y), tc::kTwoOverLn2x2)), hi.x, lo.x);
+        tc::split_bf16x2_p(tc::logistic2(tc::f2_mul(tc::f2_pack(v.z, v.w), tc::kTwoOverLn2x2)), hi.y, lo.y);
+        if (t.r < hi_row) {
+          uint32_t* sr = stage + (t.r - lo_row + (ag1 - ag0 == 2 ? t.ag * (d.stage_rows / 2) : 0)) * stage_ld;
+          *reinterpret_cast<uint2*>(sr + u0 / 2) = hi;
+          *reinterpret_cast<uint2*>(sr + H / 2 + u0 / 2) = lo;
+        }
+      };
+      Slot x, y;
+      request(x, warp);
 #pragma unroll 1
-      for (int c0 = half * (H / 2); c0 < (half + 1) * (H / 2); c0 += 16) {
-        float v[16];
-#pragma unroll
-        for (int j = 0; j < 16; j += 4) {
-          const float4 cc = __ldg(reinterpret_cast<const float4*>(cvec + c0 + j));
-          v[j] = cc.x; v[j + 1] = cc.y; v[j + 2] = cc.z; v[j + 3] = cc.w;
-        }
-#pragma unroll
-        for (int j8 = 0; j8 < 16; j8 += 8) {
-          float4 w4[10][2];
-#pragma unroll
-          for (int q = 0; q < 10; ++q) {
-            const uint32_t f = (mask >> q) & 1u ? e[q] >> 8 : 0u;
-            const float* wr = W1t + (int64_t)f * H + c0 + j8;
-            w4[q][0] = __ldg(reinterpret_cast<const float4*>(wr));
-            w4[q][1] = __ldg(reinterpret_cast<const float4*>(wr + 4));
-          }
-#pragma unroll
-          for (int q = 0; q < 10; ++q) {
-            const float dv = (mask >> q) & 1u ? (float)(int8_t)(e[q] & 0xFFu) : 0.0f;
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              float* vv = v + j8 + 4 * k;
-              vv[0] = fmaf(dv, w4[q][k].x, vv[0]);
-              vv[1] = fmaf(dv, w4[q][k].y, vv[1]);
-              vv[2] = fmaf(dv, w4[q][k].z, vv[2]);
-              vv[3] = fmaf(dv, w4[q][k].w, vv[3]);
-            }
-          }
-        }
-        uint32_t hi[8], lo[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          tc::split_bf16x2_p(tc::logistic2(tc::f2_mul(tc::f2_pack(v[2 * j], v[2 * j + 1]), tc::kTwoOverLn2x2)), hi[j], lo[j]);
-        tc::st_x8(P + c0 / 2, hi);
-        tc::st_x8(P + H / 2 + c0 / 2, lo);
+      for (int sl = warp; sl < total; sl += 16) {
+        request(y, sl + 8);
+        finish(x);
+        if (sl + 16 < total) request(x, sl + 16);
+        finish(y);
       }
-      tc::wait_st();
-      operand_ready(ag);
+    };
+    auto h1_to_tmem = [&](int ag0, int ag1, int lo_row, int hi_row) {
+      for (int ag = ag0; ag < ag1; ++ag) {
+        const int q_row = quad_row(ag);  // warps without rows of the block have nothing to move
+        if (q_row >= 0 && q_row < hi_row && q_row + 32 > lo_row) {
+          const uint32_t P = tmem + (uint32_t)(ag * 256) + lane_base;
+          const int H = d.H0, w0 = half * (H / 4);  // this half's hi words; its lo words H / 2 on
+          const uint32_t* sr =  // (lanes past the rows repeat the last one)
+              stage + (min(q_row + lane, hi_row - 1) - lo_row + (ag1 - ag0 == 2 ? ag * (d.stage_rows / 2) : 0)) * stage_ld;
+          for (int part = 0; part < 2; ++part)
+            for (int c = 0; c < H / 4; c += 16) {
+              uint32_t v[16];
+#pragma unroll
+              for (int j = 0; j < 16; j += 4) {
+                const uint4 x = *reinterpret_cast<const uint4*>(sr + part * (H / 2) + w0 + c + j);
+                v[j] = x.x, v[j + 1] = x.y, v[j + 2] = x.z, v[j + 3] = x.w;
+              }
+              tc::st_x16(P + part * (H / 2) + w0 + c, v);
+            }
+        }
+        tc::wait_st();
+      }
     };
     // epilogue 2: r2 = 1 / (1 + exp(2 (D + b2))) and this half's partial z = sum_k W3'[:, k] r2[k] on the
     // tensor cores from registers (mma.sync m16n8k16, one n-tile of 8 outputs): the warp
@@ -458,7 +513,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
       float* zp = zpart + (ag * 2 + half) * 128 * 8;
 #pragma unroll
       for (int rg = 0; rg < 2; ++rg) {
-        const int r = 32 * (warp & 3) + 16 * rg + g;
+        const int r = quad_row(ag) + 16 * rg + g;
         *reinterpret_cast<float2*>(zp + r * 8 + 2 * c4) = make_float2(zacc[rg][0], zacc[rg][1]);
         *reinterpret_cast<float2*>(zp + (r + 8) * 8 + 2 * c4) = make_float2(zacc[rg][2], zacc[rg][3]);
       }
@@ -514,38 +569,46 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
           break;
         }
       }
-      // gathered tiles: the previous step's ego rows must have left the buffer
-      if (obs_warp && t >= 1) {
-        if (!bad && !tc::mbar_wait(&obs_free, (uint32_t)(t - 1) & 1u)) bad = true;
-        bad = __any_sync(0xFFFFFFFFu, bad);
-      }
+      if (obs_warp && !boot) tc::mbar_arrive(&obs_full);  // this state's rows are in place
       // teammate first (its network runs in every step but the bootstrap)
       const int first = boot || tm_rule ? 0 : 1;
       const uint32_t par = (uint32_t)t & 1u, gt = a.step0 + (uint32_t)t;
       // this half's action draw (ego: warps 0-3, teammate: warps 4-7), ahead of its use
       const float u_act = boot ? 0.0f : u01(draw0(a.b.key, (uint32_t)my_env, gt, kStreamAct0 + half));
-      State s = st[row];  // register copy for this step (rows past count are never used)
+      // both agents' h1 in one pass where the stage holds both, else agent by agent and block
+      // of stage rows by block (a barrier before a block is written and before it is read; one
+      // more before the partial logits are written over the last)
+      if (first == 1 && 2 * count <= d.stage_rows) {
+        if (!bad) h1(0, 2, 0, count);
+        bad = sync_or();
+        if (!bad) {
+          h1_to_tmem(0, 2, 0, count);
+          operand_ready(1);
+          operand_ready(0);
+        }
+      } else {
 #pragma unroll 1
-      for (int i = first; i >= 0; --i) {
-        // the ego's u8 row is the trajectory's observation; no first layer to feed
-        if (!kXp && i == 0 && !boot && a.traj.obs && row < count)
-          Env::obs_words(a.b.env, s, 0, reinterpret_cast<uint32_t*>(sObs + row * od), my_w0, my_w1);
-        if (obs_warp && i == 0 && !boot) tc::mbar_arrive(&obs_full);
-        if (!bad) sparse_h1(i, s);
+        for (int i = first; i >= 0; --i) {
+#pragma unroll 1
+          for (int lo_row = 0; lo_row < count; lo_row += d.stage_rows) {
+            const int hi_row = min(lo_row + d.stage_rows, count);
+            if (!bad) h1(i, i + 1, lo_row, hi_row);
+            bad = sync_or();
+            if (!bad) h1_to_tmem(i, i + 1, lo_row, hi_row);
+            bad = sync_or();
+          }
+          if (!bad) operand_ready(i);
+        }
       }
+      if (!kXp && !kGather && !boot && a.traj.obs) copy_obs(t);  // overlaps L2 on the tensor cores
       if (t == a.dbg_expire_step) {  // test hook: an accumulator wait that never completes
         if (!bad && !tc::mbar_wait(&never_bar, 0, a.dbg_expire_ns)) bad = true;
         bad = __any_sync(0xFFFFFFFFu, bad);
       }
-      if (!kXp && !kGather && !boot && a.traj.obs) {  // overlaps L2 on the tensor cores
-        tc::fence_proxy_async();       // the rows were written by ordinary stores
-        if (sync_or()) break;
-        copy_obs(t);
-      }
 #pragma unroll 1
       for (int i = first; i >= 0; --i) {
         wait_acc(i, par);
-        if (!bad) epilogue2(i);
+        if (!bad && quad_row(i) >= 0 && quad_row(i) < count) epilogue2(i);
       }
       if (sync_or()) break;
       float z[16];
@@ -579,7 +642,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
           val0 = z[NA];
         }
       }
+      if (tid == 0 && bulk_obs) tc::bulk_wait_read();  // the rows may change
+      if (obs_warp && half == 0) {
+        if (!bad && !tc::mbar_wait(&obs_free, par)) bad = true;
+        bad = __any_sync(0xFFFFFFFFu, bad);
+      }
       if (sync_or()) break;
+      State s = st[row];
       if (kXp && half == 0 && row < count && alive) {
         const int act1 = act1s[row];
         const int64_t env = env0 + row;
@@ -598,6 +667,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
           if (done) alive = false;
         }
         st[row] = s;
+        put_objects(s);
       } else if (!kXp && half == 0 && row < count) {
         const int act1 = act1s[row];
         const int64_t env = my_env;
@@ -605,6 +675,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
           if (a.g.teammate) a.g.teammate[env] = tm_pol;
           if (a.g.teammate2) a.g.teammate2[env] = tm_pol;
         }
+        const State before = s;
         float r0, r1, team;
         const int done = Env::step(a.b.env, s, act0, act1, r0, r1, team);
         const int64_t o = (int64_t)t * N + env;
@@ -619,8 +690,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) ppo_tc_kernel(const PpoTcArgs a
           if (a.ep_step) a.ep_step[env] = gt + 1;
         }
         st[row] = s;
+        put_objects(s);
+        if (rows) {
+          Env::move_words(a.b.env, before, s, done > 0, reinterpret_cast<uint32_t*>(sObs + row * od));
+          if (!kGather) tc::fence_proxy_async();
+        }
       }
-      if (tid == 0 && bulk_obs) tc::bulk_wait_read();  // the rows may be rebuilt
       if (sync_or()) break;
     }
     if (tid == 0 && bulk_obs) tc::bulk_wait_all();
