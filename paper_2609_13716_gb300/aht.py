@@ -96,6 +96,8 @@ def library_path() -> str:
 def load() -> C.CDLL:
     """Loads libaht.so (built in-tree).  Raises if it is missing: no fallback exists."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = library_path()
@@ -180,6 +182,9 @@ def _check(status):
 def _ptr(t, dtype=None, shape=None, name="tensor"):
     if t is None:
         return None
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and (dtype is None or t.dtype is dtype) and \
+            (shape is None or t.shape == shape):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
@@ -193,7 +198,8 @@ def _ptr(t, dtype=None, shape=None, name="tensor"):
 
 def _stream(stream):
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the raw handle of torch.cuda.current_stream(), without building a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return getattr(stream, "cuda_stream", stream)
 
 
