@@ -137,58 +137,99 @@ cudaError_t launch_resample_group(const ResampleGroupArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// ---- GAE: one thread per env, reverse scan over T (time-major, coalesced across envs) --
-// The scan carries only two floats from step to step, so each thread loads the rewards,
-// values and done flags of kGaeChunk steps at once (independent loads in flight together)
-// and then runs the recurrence over them in the same order as a step-by-step scan.
-constexpr int kGaeChunk = 16;
+// ---- GAE: a block per 32 envs, tiles of up to 64 steps from the end of T -----------------
+// Only A_t = delta_t + (gamma lambda (1 - d_t)) A_{t+1} is sequential.  Warp w of a block
+// loads kGaeChunk steps of its 32 envs (lane = env: rows of 128 bytes), all warps at once, and
+// forms their deltas; one warp then runs the recurrence over the tile in shared memory, in the
+// order and arithmetic of a step-by-step scan; and all warps write their steps' advantages
+// and targets.  One thread per env, as before, kept too few loads in flight for the memory:
+// 16384 x 128 13.4 us, 10.1 now, against 6.6 us of traffic at 6.8 TB/s (16 steps a warp 11.8:
+// fewer warps to hide the latency; 32 warps a block 13.6).
+constexpr int kGaeChunk = 4;
+constexpr int kGaeWarps = 16;
 
-__global__ void __launch_bounds__(128) gae_kernel(const float* __restrict__ r, const float* __restrict__ v,
-                                                  const uint8_t* __restrict__ d, const float* __restrict__ v_last,
-                                                  int64_t n, int32_t T, float gamma, float lambda,
-                                                  float* __restrict__ adv, float* __restrict__ tgt) {
+__global__ void __launch_bounds__(32 * kGaeWarps, 4) gae_kernel(const float* __restrict__ r, const float* __restrict__ v,
+                                                             const uint8_t* __restrict__ d,
+                                                             const float* __restrict__ v_last, int64_t n, int32_t T,
+                                                             float gamma, float lambda, float* __restrict__ adv,
+                                                             float* __restrict__ tgt) {
+  __shared__ float s_a[kGaeWarps * kGaeChunk][32];  // delta, then the advantage
+  __shared__ float s_c[kGaeWarps * kGaeChunk][32];  // gamma lambda (1 - d)
+  __shared__ float s_v[32];                         // V of the tile's first step, for the tile before
   // launched as a programmatic dependent of the stream's previous kernel (the rollout
   // that wrote the trajectory): wait until it is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  float next_v = v_last[e];
-  float next_a = 0.0f;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile = (int)(blockDim.x >> 5) * kGaeChunk;
+  const int64_t e = blockIdx.x * (int64_t)32 + lane;
+  const bool live = e < n;
   const float gl = gamma * lambda;
-  for (int t0 = T - 1; t0 >= 0; t0 -= kGaeChunk) {
-    const int c = t0 + 1 < kGaeChunk ? t0 + 1 : kGaeChunk;  // steps t0, t0 - 1, ..., t0 - c + 1
-    float rv[kGaeChunk], vv[kGaeChunk];
+  float next_a = 0.0f;  // warp 0: A of the step after the tile
+  for (int t1 = T; t1 > 0; t1 -= tile) {  // steps [max(t1 - tile, 0), t1), row k of s_a: t1 - 1 - k
+    const int steps = min(tile, t1), k0 = warp * kGaeChunk;  // this warp's rows [k0, k0 + kGaeChunk)
+    float rv[kGaeChunk], vv[kGaeChunk + 1];  // vv[j]: V of the step after row k0 + j's
     uint8_t dv[kGaeChunk];
+    if (live && k0 < steps) {
+      // (a tile's own values are read before any of its outputs is written, so that targets may
+      // replace values in place)
+      vv[0] = t1 - k0 == T ? v_last[e] : k0 == 0 ? s_v[lane] : v[(int64_t)(t1 - k0) * n + e];
 #pragma unroll
-    for (int j = 0; j < kGaeChunk; ++j)
-      if (j < c) {
-        const int64_t i = (int64_t)(t0 - j) * n + e;
-        rv[j] = r[i];
-        vv[j] = v[i];
-        dv[j] = d[i];
-      }
+      for (int j = 0; j < kGaeChunk; ++j)
+        if (k0 + j < steps) {
+          const int64_t i = (int64_t)(t1 - 1 - k0 - j) * n + e;
+          rv[j] = r[i];
+          vv[j + 1] = v[i];
+          dv[j] = d[i];
+        }
 #pragma unroll
-    for (int j = 0; j < kGaeChunk; ++j)
-      if (j < c) {
-        const int64_t i = (int64_t)(t0 - j) * n + e;
-        const float nonterminal = dv[j] ? 0.0f : 1.0f;
-        const float delta = rv[j] + gamma * nonterminal * next_v - vv[j];
-        const float at = delta + gl * nonterminal * next_a;
-        adv[i] = at;
-        if (tgt) tgt[i] = at + vv[j];
-        next_a = at;
-        next_v = vv[j];
+      for (int j = 0; j < kGaeChunk; ++j)
+        if (k0 + j < steps) {
+          const float nonterminal = dv[j] ? 0.0f : 1.0f;
+          s_a[k0 + j][lane] = fmaf(gamma * nonterminal, vv[j], rv[j]) - vv[j + 1];
+          s_c[k0 + j][lane] = gl * nonterminal;
+        }
+    }
+    __syncthreads();
+    if (k0 + kGaeChunk == tile) s_v[lane] = vv[kGaeChunk];  // (used after a full tile only)
+    if (warp == 0) {
+      int k = 0;
+      for (; k + kGaeChunk <= steps; k += kGaeChunk) {
+        float a[kGaeChunk], c[kGaeChunk];
+#pragma unroll
+        for (int j = 0; j < kGaeChunk; ++j) a[j] = s_a[k + j][lane], c[j] = s_c[k + j][lane];
+#pragma unroll
+        for (int j = 0; j < kGaeChunk; ++j) {
+          next_a = fmaf(c[j], next_a, a[j]);
+          s_a[k + j][lane] = next_a;
+        }
       }
+      for (; k < steps; ++k) {
+        next_a = fmaf(s_c[k][lane], next_a, s_a[k][lane]);
+        s_a[k][lane] = next_a;
+      }
+    }
+    __syncthreads();
+    if (live && k0 < steps) {
+#pragma unroll
+      for (int j = 0; j < kGaeChunk; ++j)
+        if (k0 + j < steps) {
+          const int64_t i = (int64_t)(t1 - 1 - k0 - j) * n + e;
+          const float a = s_a[k0 + j][lane];
+          adv[i] = a;
+          if (tgt) tgt[i] = a + vv[j + 1];
+        }
+    }
+    __syncthreads();  // (s_a is rewritten by the next tile)
   }
 }
 
 cudaError_t launch_gae(const float* r, const float* v, const uint8_t* d, const float* v_last,
                        int64_t n, int32_t T, float gamma, float lambda, float* adv, float* tgt,
                        cudaStream_t s) {
-  const int threads = 128;  // 16384 envs -> 128 CTAs, spread over the SMs
+  const int warps = T >= kGaeWarps * kGaeChunk ? kGaeWarps : (T + kGaeChunk - 1) / kGaeChunk;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n + threads - 1) / threads));
-  cfg.blockDim = dim3(threads);
+  cfg.gridDim = dim3((unsigned)((n + 31) / 32));
+  cfg.blockDim = dim3((unsigned)(32 * warps));
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
