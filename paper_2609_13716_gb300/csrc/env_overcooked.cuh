@@ -87,51 +87,59 @@ struct EnvOvercooked {
 
   __device__ static int step(const DevEnv& d, State& s, int a0, int a1, float& r0, float& r1,
                              float& team) {
-    const bool was_cooking = s.pot_n == 3 && s.pot_timer > 0;
+    // the agents and the pot in registers (s may be in shared memory, where each byte's
+    // read-modify-write would wait for the last)
+    int ax[2] = {s.ax[0], s.ax[1]}, ay[2] = {s.ay[0], s.ay[1]};
+    int face[2] = {s.face[0], s.face[1]}, held[2] = {s.held[0], s.held[1]};
+    int pot_n = s.pot_n, pot_timer = s.pot_timer;
+    const bool was_cooking = pot_n == 3 && pot_timer > 0;
     const int act[2] = {a0, a1};
     int px[2], py[2];
+#pragma unroll
     for (int i = 0; i < 2; ++i) {
-      px[i] = s.ax[i];
-      py[i] = s.ay[i];
+      px[i] = ax[i];
+      py[i] = ay[i];
       if (act[i] >= 1 && act[i] <= 4) {
-        s.face[i] = (uint8_t)(act[i] - 1);
+        face[i] = act[i] - 1;
         int dx, dy;
-        facing(s.face[i], dx, dy);
-        if (cell(s.ax[i] + dx, s.ay[i] + dy) == 0) {
-          px[i] = s.ax[i] + dx;
-          py[i] = s.ay[i] + dy;
+        facing(face[i], dx, dy);
+        if (cell(ax[i] + dx, ay[i] + dy) == 0) {
+          px[i] = ax[i] + dx;
+          py[i] = ay[i] + dy;
         }
       }
     }
     const bool collide = (px[0] == px[1] && py[0] == py[1]) ||
-                         (px[0] == s.ax[1] && py[0] == s.ay[1] && px[1] == s.ax[0] && py[1] == s.ay[0]);
+                         (px[0] == ax[1] && py[0] == ay[1] && px[1] == ax[0] && py[1] == ay[0]);
     if (!collide) {
+#pragma unroll
       for (int i = 0; i < 2; ++i) {
-        s.ax[i] = (uint8_t)px[i];
-        s.ay[i] = (uint8_t)py[i];
+        ax[i] = px[i];
+        ay[i] = py[i];
       }
     }
     float reward = 0.0f;
+#pragma unroll
     for (int i = 0; i < 2; ++i) {
       if (act[i] != 5) continue;
       int dx, dy;
-      facing(s.face[i], dx, dy);
-      const int cx = s.ax[i] + dx, cy = s.ay[i] + dy;
+      facing(face[i], dx, dy);
+      const int cx = ax[i] + dx, cy = ay[i] + dy;
       const int c = cell(cx, cy);
-      uint8_t h = s.held[i];
+      int h = held[i];
       if (c == 2) {
         if (h == kNone) h = kOnion;
       } else if (c == 4) {
         if (h == kNone) h = kDish;
       } else if (c == 3) {
-        if (h == kOnion && s.pot_n < 3) {
+        if (h == kOnion && pot_n < 3) {
           h = kNone;
-          s.pot_n += 1;
-          if (s.pot_n == 3) s.pot_timer = (uint8_t)d.cook_time;
-        } else if (h == kDish && s.pot_n == 3 && s.pot_timer == 0) {
+          pot_n += 1;
+          if (pot_n == 3) pot_timer = (uint8_t)d.cook_time;
+        } else if (h == kDish && pot_n == 3 && pot_timer == 0) {
           h = kSoup;
-          s.pot_n = 0;
-          s.pot_timer = 0;
+          pot_n = 0;
+          pot_timer = 0;
         }
       } else if (c == 5) {
         if (h == kSoup) {
@@ -140,17 +148,27 @@ struct EnvOvercooked {
         }
       } else if (c == 1) {
         uint8_t& it = s.item[cy * 5 + cx];
-        if (h != kNone && it == kNone) {
-          it = h;
+        const int lying = it;
+        if (h != kNone && lying == kNone) {
+          it = (uint8_t)h;
           h = kNone;
-        } else if (h == kNone && it != kNone) {
-          h = it;
+        } else if (h == kNone && lying != kNone) {
+          h = lying;
           it = kNone;
         }
       }
-      s.held[i] = h;
+      held[i] = h;
     }
-    if (was_cooking && s.pot_timer > 0) s.pot_timer -= 1;
+    if (was_cooking && pot_timer > 0) pot_timer -= 1;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      s.ax[i] = (uint8_t)ax[i];
+      s.ay[i] = (uint8_t)ay[i];
+      s.face[i] = (uint8_t)face[i];
+      s.held[i] = (uint8_t)held[i];
+    }
+    s.pot_n = (uint8_t)pot_n;
+    s.pot_timer = (uint8_t)pot_timer;
     s.ep_t += 1;
     r0 = reward;
     r1 = reward;
@@ -197,15 +215,41 @@ struct EnvOvercooked {
     }
     obs_state_bits(s, seat, row);
   }
-  // The same bits into a word row (the streamed cross-play kernel): the layout and urgency
-  // channels as whole words, then the state's channels bit by bit.
+  // The same bits into a word row: every cell is a field of 26 bits at a fixed position, ORed
+  // into registers over the layout and urgency channels, one store per word (bit by bit into
+  // shared memory, each read-modify-write waited for the one before: ~2 K cycles a row).
   __device__ static void obs_into(const DevEnv& d, const State& s, int seat, ObsBits& row) {
     constexpr OcObsMasks M = oc_obs_masks();
     const uint32_t u = urgent(d, s) ? 0xFFFFFFFFu : 0u;
+    uint32_t wd[kOcObsWords];
 #pragma unroll
-    for (int i = 0; i < kOcObsWords; ++i) row.w[i] = M.layout[i] | (M.urgent[i] & u);
+    for (int i = 0; i < kOcObsWords; ++i) wd[i] = M.layout[i] | (M.urgent[i] & u);
+    int at[2];            // the agents' cells: self, the other
+    uint32_t agent[2];    // and their bits there
+#pragma unroll
+    for (int who = 0; who < 2; ++who) {
+      const bool first = (who == 0) == (seat == 0);  // agent 0
+      const int ax = first ? s.ax[0] : s.ax[1], ay = first ? s.ay[0] : s.ay[1];
+      const int face = first ? s.face[0] : s.face[1], held = first ? s.held[0] : s.held[1];
+      at[who] = ay * 5 + ax;
+      agent[who] = (1u << who) | (1u << (2 + 4 * who + face)) |
+                   (held != kNone ? (1u << (23 + who)) | (1u << (14 + held)) : 0u);
+    }
+    const uint32_t pot = (s.pot_n >= 1 ? 1u << (17 + s.pot_n) : 0u) |
+                         (s.pot_n == 3 ? (s.pot_timer > 0 ? 1u << 21 : 1u << 22) : 0u);
+#pragma unroll
+    for (int c = 0; c < 20; ++c) {
+      const int t = kitchen_type(c);
+      uint32_t v = (at[0] == c ? agent[0] : 0u) | (at[1] == c ? agent[1] : 0u);
+      if (t == 1) v |= s.item[c] != kNone ? 1u << (14 + s.item[c]) : 0u;
+      if (t == 3) v |= pot;
+      const int w = (26 * c) >> 5, sh = (26 * c) & 31;
+      wd[w] |= v << sh;
+      if (sh + 26 > 32) wd[w + 1] |= v >> (32 - sh);
+    }
+#pragma unroll
+    for (int i = 0; i < kOcObsWords; ++i) row.w[i] = wd[i];
     for (int i = kOcObsWords; i < row.words; ++i) row.w[i] = 0u;
-    obs_state_bits(s, seat, row);
   }
   __device__ static void obs(const DevEnv& d, const State& s, int seat, uint8_t* row) {
     ObsBytes w{row, 130};
