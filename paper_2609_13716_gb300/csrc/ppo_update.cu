@@ -10,9 +10,9 @@
 // the working accumulator 128: 496 of 512) and leave once, as the CTA's partial sum.  Operands live in shared memory as rows of samples (8 x 16-byte core matrices, 8
 // samples x 8 features): the same buffer is the K-major A operand of a forward product
 // (samples as M) and the MN-major operand of a weight-gradient product (samples as K).
-// Forward products run with M = 128 over a 64-sample tile: the upper 64 rows read the
-// next buffer in shared memory and their accumulator lanes are never read.  Activations
-// and gradients are split into two bf16 (x = hi + lo, ~2^-17 relative); W1, W2 are bf16.
+// Forward and backward products run with M = 64, whose 64 rows are the first 16
+// tensor-memory lanes of every warp quadrant.  Activations and gradients are split into two
+// bf16 (x = hi + lo, ~2^-17 relative); W1, W2 are bf16.
 #include <cfloat>
 
 #include "kernels.h"
@@ -27,13 +27,20 @@ constexpr int kKP = kPpoKP;          // padded input width: obs + the bias colum
 constexpr int kH = kPpoHidden;       // hidden width
 constexpr int kH1P = 144;            // h1 row width as the B operand of dW2 (+ ones + pad)
 constexpr int kNO = 8;               // output rows (actions + value), padded
-// Warps w with w % 4 in {0, 1} reach tensor-memory lanes 0..63 (the tile's samples): the 8
-// compute warps 0, 1, 4, 5, 8, 9, 12, 13 (four threads per sample, 32 features each).
-// Warp 2 issues the MMAs; warps 3, 6, 7 and 10 load the next tile; warp 11 idles.
-constexpr int kThreadsPpo = 448;
-constexpr int kCompute = 256;
+// A tile is a chain of five products with an epilogue after each, so what bounds the kernel
+// is the epilogues' issue rate and the hand-over between them.  Sixteen compute warps, four
+// per scheduler: warp w takes the 16 samples of quadrant w % 4 and the 32 features of group
+// w / 4, as the 8 x 8 fragments that 16-lane tensor-memory loads, ldmatrix and stmatrix
+// share.  (With M = 128 over the tile's 64 rows only the warps of two schedulers could reach
+// the results: 10.3 against 8.4 ms for 4 epochs x 4 minibatches of 2 M samples.)
+constexpr int kComputeWarps = 16;
+constexpr int kCompute = 32 * kComputeWarps;
+constexpr int kMmaWarp = kComputeWarps;          // issues the MMAs
+constexpr int kLoadWarp = kComputeWarps + 1;     // four warps that load the next tile
 constexpr int kLoaders = 128;
+constexpr int kThreadsPpo = kCompute + 32 + kLoaders;
 constexpr int kComputeBar = 1;
+constexpr int kWarpCols = kH / (kComputeWarps / 4);  // features per compute warp
 
 // shared memory (bytes from the 1024-aligned base)
 constexpr uint32_t kOffX = 0;                                  // [64][208] bf16
@@ -50,11 +57,6 @@ constexpr uint32_t kOffSC = kOffPK + kPpoPackedBytes;          // [2][5][64] per
 constexpr uint32_t kSmemUsed = kOffSC + 2 * 5 * kRows * 4;
 constexpr uint32_t kOffRed = kOffDA2hi;                        // [64][16] f32 end-of-kernel sums
 static_assert(kOffH1hi == 26624 && kOffPK == 133120, "layout");
-// every M = 128 A operand of a 64-sample buffer reads 64 more rows from what follows
-static_assert(kOffX + 2 * kRows * kKP * 2 <= kSmemUsed && kOffDA2lo + 2 * kRows * kH * 2 <= kSmemUsed &&
-                  kOffH2lo + 2 * kRows * kH * 2 <= kSmemUsed && kOffDZlo + 2 * kRows * 16 * 2 <= kSmemUsed,
-              "A operands stay inside shared memory");
-
 // tensor memory columns
 constexpr uint32_t kTmAcc = 0, kTmDW1 = 128, kTmDW2 = 336, kTmDW3 = 480;
 
@@ -88,6 +90,20 @@ __device__ __forceinline__ void unpack_bf16x2(uint32_t v, float& a, float& b) {
   b = __uint_as_float(v & 0xFFFF0000u);
 }
 
+// Four 8 x 8 bf16 matrices between shared memory and fragments: lane 8m + r holds the address
+// of row r of matrix m (16 bytes); a lane's words are row lane / 4, columns 2 (lane % 4), + 1.
+__device__ __forceinline__ void ld_matrix_x4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void st_matrix_x4(uint32_t addr, const uint32_t (&r)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+
 // f32 pair (x0, x1) -> hi | lo bf16 pairs
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
   tc::split_bf16x2_p(tc::f2_pack(x0, x1), hi, lo);
@@ -117,8 +133,8 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
 
   if (tid == 0) {
     for (int i = 0; i < 6; ++i) {
-      // X: the loader warps; dz: the 64 threads that compute the sample's loss
-      tc::mbar_init(&opnd_bar[i], i == kX ? kLoaders : (i == kDZ ? kRows : kCompute));
+      // X: the loader warps; dz: the four warps that compute the samples' losses
+      tc::mbar_init(&opnd_bar[i], i == kX ? kLoaders : (i == kDZ ? 128 : kCompute));
       tc::mbar_init(&acc_bar[i], 1);
     }
     tc::mbar_init(&wload_bar, 1);
@@ -143,16 +159,16 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
   tc::fence_after_sync();
   const uint32_t tmem = tmem_slot;
 
-  if (warp == 2) {
+  if (warp == kMmaWarp) {
     // ================================ MMA warp =====================================
     if (lane == 0 && n_it > 0) {
       tc::mbar_expect_tx(&wload_bar, kPpoPackedBytes);
       for (uint32_t off = 0; off < kPpoPackedBytes; off += 32768u)
         tc::bulk_g2s(sm + kOffPK + off, a.packed + off, min(32768u, kPpoPackedBytes - off), &wload_bar);
       bool ok = tc::mbar_wait(&wload_bar, 0);
-      const uint32_t idL = tc::idesc_bf16(128, kH);                               // L1, L2
-      const uint32_t idZ = tc::idesc_bf16(128, 16);                               // logits
-      const uint32_t idH = tc::idesc_bf16(128, kH) | (1u << 16);                  // B MN-major
+      const uint32_t idL = tc::idesc_bf16(kRows, kH);                             // L1, L2
+      const uint32_t idZ = tc::idesc_bf16(kRows, 16);                             // logits
+      const uint32_t idH = tc::idesc_bf16(kRows, kH) | (1u << 16);                // B MN-major
       const uint32_t id3 = tc::idesc_bf16(128, 16) | (1u << 15) | (1u << 16);     // dW3^T
       const uint32_t id2 = tc::idesc_bf16(128, kH1P) | (1u << 15) | (1u << 16);   // dW2
       const uint32_t id1 = tc::idesc_bf16(128, kKP) | (1u << 15) | (1u << 16);    // dW1
@@ -247,9 +263,9 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       }
       if (!ok) abort_flag = 1;
     }
-  } else if (warp == 3 || warp == 6 || warp == 7 || warp == 10) {
+  } else if (warp >= kLoadWarp) {
     // =============================== loader warps ===================================
-    // Loader k (warps 3, 6, 7, 10) owns rows 16k .. 16k + 15 of every tile, two lanes per
+    // Loader k owns rows 16k .. 16k + 15 of every tile, two lanes per
     // row (words 26h .. 26h + 25 of the observation row for lane half h): it draws the
     // sample from the permutation and loads its observation words and scalars one tile
     // ahead, into registers; once the previous tile's last MMA has completed it writes
@@ -259,8 +275,7 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     // cycles, measured), and epilogue 2 suffers least.
     if (n_it > 0) {
       const int D = a.D, nw = D / 4;
-      const int li = warp == 3 ? 0 : (warp == 6 ? 1 : (warp == 7 ? 2 : 3));
-      const int row = li * 16 + (lane >> 1), hw = lane & 1;
+      const int row = (warp - kLoadWarp) * 16 + (lane >> 1), hw = lane & 1;
       constexpr int kHalfWords = kKP / 8;   // 26 words per lane
       const float mu = a.mbstat[0], inv_sd = a.mbstat[1];
       uint32_t ow[kHalfWords];
@@ -307,12 +322,19 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       }
       if (!ok) abort_flag = 1;
     }
-  } else if ((warp & 2) == 0) {
+  } else {
     // ============================== compute warps ===================================
-    const int quarter = warp >> 2;                                 // features 32q .. 32q + 31
-    const int row = (warp & 1) * 32 + lane;                       // sample row of the tile
-    const int c0 = quarter * 32;
-    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;  // tensor-memory lanes
+    const int quad = warp & 3, c0 = (warp >> 2) * kWarpCols;      // samples 16 quad .., features c0 ..
+    const int c2 = 2 * (lane & 3);                                // this lane's feature pair of a block of 8
+    const uint32_t lane_base = (uint32_t)(quad * 32) << 16;       // tensor-memory lanes
+    // the loss: lanes 0..15 of the first group's warps hold one sample each
+    const bool loss_warp = warp < 4;
+    const int row = quad * 16 + (lane & 15);
+    // this lane's matrix row of the 16 samples x 8 features at column 0: matrices 0, 1 are the
+    // hi rows 0..7 and 8..15, matrices 2, 3 the lo rows
+    auto frag_addr = [&](uint32_t hi, uint32_t lo, int W) {
+      return base + (lane & 16 ? lo : hi) + canon(quad * 16 + (lane & 15), 0, W);
+    };
     const int A = a.n_act;
     const float eps = a.clip_eps, inv_b = 1.0f / (float)a.B;
     const float* b1 = reinterpret_cast<const float*>(pk + kPkB1);
@@ -331,74 +353,78 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       tc::fence_before_sync();
       tc::mbar_arrive(&opnd_bar[i]);
     };
-    auto sync_or = [&]() { return tc::bar_or(kComputeBar, kCompute, bad || abort_flag); };
-    // tanh(acc + bias) of this thread's 32 columns -> hi | lo bf16 rows at dst (row width W)
-    auto act_rows = [&](const float* bias, uint32_t dst_hi, uint32_t dst_lo, int W) {
-      uint32_t v[32];
-      tc::ld_x32(tmem + kTmAcc + lane_base + c0, v);
+    // the accumulator's 16 samples x 32 features, as fragments of 8 features
+    auto acc_frags = [&](uint32_t (&v)[kWarpCols / 8][4]) {
+#pragma unroll
+      for (int b = 0; b < kWarpCols / 8; ++b) tc::ld_16x256b(tmem + kTmAcc + lane_base + c0 + 8 * b, v[b]);
       tc::wait_ld();
-      uint32_t hi[16], lo[16];
+    };
+    // tanh(acc + bias) -> hi | lo bf16 rows at dst (row width W)
+    auto act_rows = [&](const float* bias, uint32_t dst_hi, uint32_t dst_lo, int W) {
+      const uint32_t dst = frag_addr(dst_hi, dst_lo, W) + (uint32_t)c0 * 16u;
+      uint64_t bb[kWarpCols / 8];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const uint64_t x = tc::f2_add(tc::f2_pack(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1])),
-                                      tc::f2_pack(bias[c0 + 2 * q], bias[c0 + 2 * q + 1]));
-        tc::split_bf16x2_p(tc::tanh2(x), hi[q], lo[q]);
-      }
+      for (int b = 0; b < kWarpCols / 8; ++b)
+        bb[b] = *reinterpret_cast<const uint64_t*>(bias + c0 + 8 * b + c2);
+      uint32_t v[kWarpCols / 8][4];
+      acc_frags(v);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        *reinterpret_cast<uint4*>(sm + dst_hi + canon(row, c0 + 8 * q, W)) =
-            make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
-        *reinterpret_cast<uint4*>(sm + dst_lo + canon(row, c0 + 8 * q, W)) =
-            make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
+      for (int b = 0; b < kWarpCols / 8; ++b) {
+        uint32_t o[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          tc::split_bf16x2_p(
+              tc::tanh2(tc::f2_add(tc::f2_pack(__uint_as_float(v[b][2 * h]), __uint_as_float(v[b][2 * h + 1])), bb[b])),
+              o[h], o[2 + h]);
+        st_matrix_x4(dst + 128u * b, o);
       }
     };
     // g (1 - h^2), h = hi + lo from the rows at src (row width W), -> hi | lo rows at dst
     auto grad_rows = [&](uint32_t src_hi, uint32_t src_lo, int W, uint32_t dst_hi, uint32_t dst_lo) {
-      uint32_t v[32];
-      tc::ld_x32(tmem + kTmAcc + lane_base + c0, v);
-      tc::wait_ld();
+      const uint32_t src = frag_addr(src_hi, src_lo, W) + (uint32_t)c0 * 16u;
+      const uint32_t dst = frag_addr(dst_hi, dst_lo, kH) + (uint32_t)c0 * 16u;
+      uint32_t v[kWarpCols / 8][4];
+      acc_frags(v);
 #pragma unroll
-      for (int q8 = 0; q8 < 4; ++q8) {
-        const int c = c0 + 8 * q8;
-        const uint4 hh = *reinterpret_cast<const uint4*>(sm + src_hi + canon(row, c, W));
-        const uint4 hl = *reinterpret_cast<const uint4*>(sm + src_lo + canon(row, c, W));
-        const uint32_t hv[4] = {hh.x, hh.y, hh.z, hh.w}, lv4[4] = {hl.x, hl.y, hl.z, hl.w};
-        uint32_t dh[4], dl[4];
+      for (int b = 0; b < kWarpCols / 8; ++b) {
+        uint32_t hv[4], o[4];
+        ld_matrix_x4(src + 128u * b, hv);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int h2 = 0; h2 < 2; ++h2) {
           float h0a, h0b, h1a, h1b;
-          unpack_bf16x2(hv[q], h0a, h1a);
-          unpack_bf16x2(lv4[q], h0b, h1b);
+          unpack_bf16x2(hv[h2], h0a, h1a);
+          unpack_bf16x2(hv[2 + h2], h0b, h1b);
           const uint64_t h = tc::f2_add(tc::f2_pack(h0a, h1a), tc::f2_pack(h0b, h1b));
           const uint64_t one_m = tc::f2_fma(h, tc::f2_sub(0ull, h), tc::f2_pack(1.0f, 1.0f));  // 1 - h^2
-          const uint64_t g = tc::f2_pack(__uint_as_float(v[8 * q8 + 2 * q]), __uint_as_float(v[8 * q8 + 2 * q + 1]));
-          tc::split_bf16x2_p(tc::f2_mul(g, one_m), dh[q], dl[q]);
+          const uint64_t g = tc::f2_pack(__uint_as_float(v[b][2 * h2]), __uint_as_float(v[b][2 * h2 + 1]));
+          tc::split_bf16x2_p(tc::f2_mul(g, one_m), o[h2], o[2 + h2]);
         }
-        *reinterpret_cast<uint4*>(sm + dst_hi + canon(row, c, kH)) = make_uint4(dh[0], dh[1], dh[2], dh[3]);
-        *reinterpret_cast<uint4*>(sm + dst_lo + canon(row, c, kH)) = make_uint4(dl[0], dl[1], dl[2], dl[3]);
+        st_matrix_x4(dst + 128u * b, o);
       }
     };
+    // A wait that ran out ends this warp's loop; the others' waits then run out as well (each
+    // is bounded) and all meet again below.
 
     for (int it = 0; it < n_it; ++it) {
       const uint32_t par = (uint32_t)it & 1u;
       // the loader wrote this tile's X and scalars, after the previous tile's last MMA:
       // every operand buffer is free again
       if (!bad && !tc::mbar_wait(&opnd_bar[kX], par)) bad = true;
-      if (sync_or()) { bad = true; break; }
       // ---- epilogue 1: h1 = tanh(acc + b1) -> hi | lo rows -------------------------
       wait_acc(kL1, par);
-      if (sync_or()) { bad = true; break; }   // every compute thread leaves at the same point
+      if (bad) break;
       act_rows(b1, kOffH1hi, kOffH1lo, kH1P);
       release(kH1);
       // ---- epilogue 2: h2 = tanh(acc + b2) -> hi | lo rows -------------------------
       wait_acc(kL2, par);
-      if (sync_or()) { bad = true; break; }
+      if (bad) break;
       act_rows(b2, kOffH2hi, kOffH2lo, kH);
       release(kH2);
-      // ---- the sample's loss and dL/dz (quarter 0, one thread per sample) -----------
-      wait_acc(kZ, par);
-      if (sync_or()) { bad = true; break; }
-      if (quarter == 0) {
+      // ---- the sample's loss and dL/dz (one lane per sample; lanes 16.. compute on
+      // accumulator lanes that no product writes, and store nothing) ------------------
+      if (loss_warp) {
+        wait_acc(kZ, par);
+        if (bad) break;
         const float* sc = reinterpret_cast<const float*>(sm + kOffSC) + (it & 1) * 5 * kRows;
         const int act = __float_as_int(sc[row]);
         const float lp_old = sc[kRows + row], v_old = sc[2 * kRows + row];
@@ -459,28 +485,30 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
           dzsum[2 * q + 1] += dz[2 * q + 1];
           split2(dz[2 * q], dz[2 * q + 1], zh[q], zl[q]);
         }
-        *reinterpret_cast<uint4*>(sm + kOffDZhi + canon(row, 0, 16)) = make_uint4(zh[0], zh[1], zh[2], zh[3]);
-        *reinterpret_cast<uint4*>(sm + kOffDZlo + canon(row, 0, 16)) = make_uint4(zl[0], zl[1], zl[2], zl[3]);
+        if (lane < 16) {
+          *reinterpret_cast<uint4*>(sm + kOffDZhi + canon(row, 0, 16)) = make_uint4(zh[0], zh[1], zh[2], zh[3]);
+          *reinterpret_cast<uint4*>(sm + kOffDZlo + canon(row, 0, 16)) = make_uint4(zl[0], zl[1], zl[2], zl[3]);
+        }
         release(kDZ);
       }
       // ---- dL/da2 = (dz W3) (1 - h2^2) --------------------------------------------
       wait_acc(kDH2, par);
-      if (sync_or()) { bad = true; break; }
+      if (bad) break;
       grad_rows(kOffH2hi, kOffH2lo, kH, kOffDA2hi, kOffDA2lo);
       release(kDA2);
       // ---- epilogue 3: dL/da1 = (da2 W2) (1 - h1^2) into the h2 rows ----------------
       wait_acc(kDH1, par);
-      if (sync_or()) { bad = true; break; }
+      if (bad) break;
       grad_rows(kOffH1hi, kOffH1lo, kH1P, kOffH2hi, kOffH2lo);
       release(kDA1);
     }
     if (n_it > 0 && !bad) wait_acc(kDW1, (uint32_t)(n_it - 1) & 1u);  // the last dW1 (all MMAs)
     if (bad) abort_flag = 1;
-    // per-CTA sums over the quarter-0 threads: dz (db3) and the loss diagnostics, row order
+    // per-CTA sums over the samples' lanes: dz (db3) and the loss diagnostics, row order
     __syncwarp();
     tc::bar_or(kComputeBar, kCompute, false);
     float* red = reinterpret_cast<float*>(sm + kOffRed);  // [64][16]
-    if (quarter == 0) {
+    if (loss_warp && lane < 16) {
 #pragma unroll
       for (int o = 0; o < kNO; ++o) red[row * 16 + o] = dzsum[o];
       red[row * 16 + 8] = st_loss;
@@ -546,7 +574,7 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
   tc::fence_before_sync();
   __syncthreads();
   if (tid == 0 && abort_flag) atomicOr(a.status, kStatusTimeout);
-  if (warp == 2 && lane == 0) {
+  if (warp == kMmaWarp && lane == 0) {
     tc::commit(&drain_bar);
     tc::mbar_wait(&drain_bar, 0);
   }
