@@ -133,8 +133,8 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
 
   if (tid == 0) {
     for (int i = 0; i < 6; ++i) {
-      // X: the loader warps; dz: the four warps that compute the samples' losses
-      tc::mbar_init(&opnd_bar[i], i == kX ? kLoaders : (i == kDZ ? 128 : kCompute));
+      // X: the loader warps; dz: the eight warps that compute the samples' losses
+      tc::mbar_init(&opnd_bar[i], i == kX ? kLoaders : (i == kDZ ? 256 : kCompute));
       tc::mbar_init(&acc_bar[i], 1);
     }
     tc::mbar_init(&wload_bar, 1);
@@ -265,36 +265,42 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     }
   } else if (warp >= kLoadWarp) {
     // =============================== loader warps ===================================
-    // Loader k owns rows 16k .. 16k + 15 of every tile, two lanes per
-    // row (words 26h .. 26h + 25 of the observation row for lane half h): it draws the
-    // sample from the permutation and loads its observation words and scalars one tile
-    // ahead, into registers; once the previous tile's last MMA has completed it writes
-    // them out as the X operand (feature D is the constant 1 that carries db1 through
-    // dW1) and the scalar rows, and releases the tile.  The next tile's loads are issued
-    // once epilogue 1 is over: the loads slow whatever epilogue they overlap (~1-1.5 K
-    // cycles, measured), and epilogue 2 suffers least.
+    // Loader k owns rows 16k .. 16k + 15 of every tile: lane r draws the sample of row r from
+    // the permutation and loads its scalars; the observation words go 8 rows x 4 consecutive
+    // words to a load (a load then touches 8 lines; a row or half a row per lane touched 32,
+    // and the L1's passes over them held up the epilogues' shared-memory accesses by 1-1.5 K
+    // cycles a tile).  Everything is loaded one tile ahead, into registers; once the previous
+    // tile's last MMA has completed the words are written out as the X operand (feature D is
+    // the constant 1 that carries db1 through dW1), 16 lanes to a core matrix, with the scalar
+    // rows, and the tile is released.  The next tile's loads are issued once epilogue 1 is
+    // over.
     if (n_it > 0) {
       const int D = a.D, nw = D / 4;
-      const int row = (warp - kLoadWarp) * 16 + (lane >> 1), hw = lane & 1;
-      constexpr int kHalfWords = kKP / 8;   // 26 words per lane
+      const int row0 = (warp - kLoadWarp) * 16;
+      const int rr = (lane >> 1) & 7, w0 = 2 * (lane >> 4) + (lane & 1);  // row of 8, word of 4
+      constexpr int kQuads = kKP / 16;      // 13 groups of 4 words per row
       const float mu = a.mbstat[0], inv_sd = a.mbstat[1];
-      uint32_t ow[kHalfWords];
+      uint32_t ow[2][kQuads];
       float sc[5];
       auto load_tile = [&](int it) {
-        const uint32_t j = a.mb * a.B + (uint32_t)(t0 + it) * kRows + (uint32_t)row;
-        const uint32_t smp = perm_index(a.key, a.epoch, a.w, a.S, j);
-        const uint32_t* orow = reinterpret_cast<const uint32_t*>(a.obs + (size_t)smp * D);
+        const uint32_t j = a.mb * a.B + (uint32_t)(t0 + it) * kRows + (uint32_t)(row0 + (lane & 15));
+        const uint32_t mine = perm_index(a.key, a.epoch, a.w, a.S, j);
 #pragma unroll
-        for (int q0 = 0; q0 < kHalfWords; ++q0) {
-          const int q = hw * kHalfWords + q0;
-          ow[q0] = q < nw ? __ldg(orow + q) : (q == nw ? 1u : 0u);
+        for (int t = 0; t < 2; ++t) {
+          const uint32_t smp = __shfl_sync(0xFFFFFFFFu, mine, 8 * t + rr);
+          const uint32_t* orow = reinterpret_cast<const uint32_t*>(a.obs + (size_t)smp * D);
+#pragma unroll
+          for (int k = 0; k < kQuads; ++k) {
+            const int q = 4 * k + w0;
+            ow[t][k] = q < nw ? __ldg(orow + q) : (q == nw ? 1u : 0u);
+          }
         }
-        if (hw == 0) {
-          sc[0] = __int_as_float((int)a.act[smp]);
-          sc[1] = a.logp[smp];
-          sc[2] = a.val[smp];
-          sc[3] = (a.adv[smp] - mu) * inv_sd;
-          sc[4] = a.tgt[smp];
+        if (lane < 16) {
+          sc[0] = __int_as_float((int)a.act[mine]);
+          sc[1] = a.logp[mine];
+          sc[2] = a.val[mine];
+          sc[3] = (a.adv[mine] - mu) * inv_sd;
+          sc[4] = a.tgt[mine];
         }
       };
       bool ok = true;
@@ -305,18 +311,18 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         if (!ok) break;
         float* scw = reinterpret_cast<float*>(sm + kOffSC) + (it & 1) * 5 * kRows;
 #pragma unroll
-        for (int c = 0; c < kHalfWords / 2; ++c)
-          *reinterpret_cast<uint4*>(sm + kOffX + canon(row, 8 * (hw * kHalfWords / 2 + c), kKP)) =
-              make_uint4(tc::bytes_to_bf16x2(ow[2 * c], 0), tc::bytes_to_bf16x2(ow[2 * c], 2),
-                         tc::bytes_to_bf16x2(ow[2 * c + 1], 0), tc::bytes_to_bf16x2(ow[2 * c + 1], 2));
-        if (hw == 0) {
+        for (int t = 0; t < 2; ++t)
 #pragma unroll
-          for (int k = 0; k < 5; ++k) scw[k * kRows + row] = sc[k];
+          for (int k = 0; k < kQuads; ++k)
+            *reinterpret_cast<uint2*>(sm + kOffX + canon(row0 + 8 * t + rr, 16 * k + 4 * w0, kKP)) =
+                make_uint2(tc::bytes_to_bf16x2(ow[t][k], 0), tc::bytes_to_bf16x2(ow[t][k], 2));
+        if (lane < 16) {
+#pragma unroll
+          for (int k = 0; k < 5; ++k) scw[k * kRows + row0 + lane] = sc[k];
         }
         tc::fence_proxy_async();
         tc::mbar_arrive(&opnd_bar[kX]);
         if (it + 1 < n_it) {
-          if (ok) ok = tc::mbar_wait(&acc_bar[kL2], (uint32_t)it & 1u);  // epilogue 1 is over
           load_tile(it + 1);
         }
       }
@@ -327,9 +333,9 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     const int quad = warp & 3, c0 = (warp >> 2) * kWarpCols;      // samples 16 quad .., features c0 ..
     const int c2 = 2 * (lane & 3);                                // this lane's feature pair of a block of 8
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;       // tensor-memory lanes
-    // the loss: lanes 0..15 of the first group's warps hold one sample each
-    const bool loss_warp = warp < 4;
-    const int row = quad * 16 + (lane & 15);
+    // the loss: the sample of this lane
+    const bool loss_warp = warp < 8;
+    const int row = quad * 16 + 8 * (warp >> 2 & 1) + (lane >> 2);
     // this lane's matrix row of the 16 samples x 8 features at column 0: matrices 0, 1 are the
     // hi rows 0..7 and 8..15, matrices 2, 3 the lo rows
     auto frag_addr = [&](uint32_t hi, uint32_t lo, int W) {
@@ -342,7 +348,7 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     const float* b3 = reinterpret_cast<const float*>(pk + kPkB3);
     bool bad = n_it > 0 && !tc::mbar_wait(&wload_bar, 0);
     float st_loss = 0.f, st_pg = 0.f, st_v = 0.f, st_ent = 0.f, st_kl = 0.f, st_clip = 0.f;
-    float dzsum[kNO] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float dzsum[2] = {0.f, 0.f};
     auto wait_acc = [&](int i, uint32_t par) {
       if (!bad && !tc::mbar_wait(&acc_bar[i], par)) bad = true;
       bad = __any_sync(0xFFFFFFFFu, bad);
@@ -420,57 +426,64 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       if (bad) break;
       act_rows(b2, kOffH2hi, kOffH2lo, kH);
       release(kH2);
-      // ---- the sample's loss and dL/dz (one lane per sample; lanes 16.. compute on
-      // accumulator lanes that no product writes, and store nothing) ------------------
+      // ---- the samples' losses and dL/dz: four lanes to a sample, two outputs each (the
+      // fragment of the 8 output columns); the first group's warps take the quadrant's samples
+      // 0..7, the second's 8..15 ---------------------------------------------------------
       if (loss_warp) {
-        wait_acc(kZ, par);
-        if (bad) break;
         const float* sc = reinterpret_cast<const float*>(sm + kOffSC) + (it & 1) * 5 * kRows;
         const int act = __float_as_int(sc[row]);
         const float lp_old = sc[kRows + row], v_old = sc[2 * kRows + row];
         const float adv_n = sc[3 * kRows + row], ret = sc[4 * kRows + row];
-        uint32_t zr[16];
-        tc::ld_x16(tmem + kTmAcc + lane_base, zr);
+        wait_acc(kZ, par);
+        if (bad) break;
+        uint32_t zr[4];
+        tc::ld_16x256b(tmem + kTmAcc + lane_base, zr);
         tc::wait_ld();
-        float z[kNO];
-#pragma unroll
-        for (int o = 0; o < kNO; ++o) z[o] = __uint_as_float(zr[o]) + b3[o];
+        const float z[2] = {__uint_as_float(warp < 4 ? zr[0] : zr[2]) + b3[c2],
+                            __uint_as_float(warp < 4 ? zr[1] : zr[3]) + b3[c2 + 1]};
+        auto sum4 = [&](float x) {  // over a sample's four lanes
+          x += __shfl_xor_sync(0xFFFFFFFFu, x, 1);
+          return x + __shfl_xor_sync(0xFFFFFFFFu, x, 2);
+        };
         // log-softmax, entropy, ratio, clipped surrogate, clipped value loss
-        float mx = -FLT_MAX;
-#pragma unroll
-        for (int o = 0; o < kNO; ++o)
-          if (o < A) mx = fmaxf(mx, z[o]);
-        float se = 0.f;
-#pragma unroll
-        for (int o = 0; o < kNO; ++o)
-          if (o < A) se += __expf(z[o] - mx);
+        float mx = fmaxf(c2 < A ? z[0] : -FLT_MAX, c2 + 1 < A ? z[1] : -FLT_MAX);
+        mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
+        const float se = sum4((c2 < A ? __expf(z[0] - mx) : 0.f) + (c2 + 1 < A ? __expf(z[1] - mx) : 0.f));
         const float lse = mx + __logf(se);
-        float logp[kNO], prob[kNO], ent = 0.f, lp_a = 0.f;
+        float logp[2], prob[2], ent_l = 0.f, lp_l = 0.f, v_l = 0.f;
 #pragma unroll
-        for (int o = 0; o < kNO; ++o) {
-          logp[o] = z[o] - lse;
-          prob[o] = o < A ? __expf(logp[o]) : 0.f;
-          if (o < A) ent -= prob[o] * logp[o];
-          if (o == act) lp_a = logp[o];
+        for (int k = 0; k < 2; ++k) {
+          const int o = c2 + k;
+          logp[k] = z[k] - lse;
+          prob[k] = o < A ? __expf(logp[k]) : 0.f;
+          if (o < A) ent_l -= prob[k] * logp[k];
+          if (o == act) lp_l = logp[k];
+          if (o == A) v_l = z[k];
         }
+        const float lp_a = sum4(lp_l), V = sum4(v_l), ent = sum4(ent_l);
         const float rho = __expf(lp_a - lp_old);
         const float rho_c = fminf(fmaxf(rho, 1.0f - eps), 1.0f + eps);
         const float un = rho * adv_n, cl = rho_c * adv_n;
         const float g_rho = un <= cl ? -adv_n : 0.0f;
-        float V = 0.f;
-#pragma unroll
-        for (int o = 0; o < kNO; ++o)
-          if (o == A) V = z[o];
         const float vc = v_old + fminf(fmaxf(V - v_old, -eps), eps);
         const float u = V - ret, w = vc - ret;
         const float dV = u * u >= w * w ? u : 0.0f;
-        float dz[kNO];
+        float dz[2];
 #pragma unroll
-        for (int o = 0; o < kNO; ++o) {
-          const float pol = g_rho * rho * ((o == act ? 1.0f : 0.0f) - prob[o]) +
-                            a.ent_coef * prob[o] * (logp[o] + ent);
-          dz[o] = o < A ? pol * inv_b : (o == A ? a.vf_coef * dV * inv_b : 0.0f);
+        for (int k = 0; k < 2; ++k) {
+          const int o = c2 + k;
+          const float pol = g_rho * rho * ((o == act ? 1.0f : 0.0f) - prob[k]) +
+                            a.ent_coef * prob[k] * (logp[k] + ent);
+          dz[k] = o < A ? pol * inv_b : (o == A ? a.vf_coef * dV * inv_b : 0.0f);
         }
+        uint32_t zh, zl;
+        split2(dz[0], dz[1], zh, zl);
+        *reinterpret_cast<uint32_t*>(sm + kOffDZhi + canon(row, c2, 16)) = zh;
+        *reinterpret_cast<uint32_t*>(sm + kOffDZlo + canon(row, c2, 16)) = zl;
+        release(kDZ);
+        dzsum[0] += dz[0];
+        dzsum[1] += dz[1];
         const float pg = -fminf(un, cl), lv = 0.5f * fmaxf(u * u, w * w);
         st_loss += pg + a.vf_coef * lv - a.ent_coef * ent;
         st_pg += pg;
@@ -478,18 +491,6 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         st_ent += ent;
         st_kl += lp_old - lp_a;
         st_clip += fabsf(rho - 1.0f) > eps ? 1.0f : 0.0f;
-        uint32_t zh[4], zl[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          dzsum[2 * q] += dz[2 * q];
-          dzsum[2 * q + 1] += dz[2 * q + 1];
-          split2(dz[2 * q], dz[2 * q + 1], zh[q], zl[q]);
-        }
-        if (lane < 16) {
-          *reinterpret_cast<uint4*>(sm + kOffDZhi + canon(row, 0, 16)) = make_uint4(zh[0], zh[1], zh[2], zh[3]);
-          *reinterpret_cast<uint4*>(sm + kOffDZlo + canon(row, 0, 16)) = make_uint4(zl[0], zl[1], zl[2], zl[3]);
-        }
-        release(kDZ);
       }
       // ---- dL/da2 = (dz W3) (1 - h2^2) --------------------------------------------
       wait_acc(kDH2, par);
@@ -508,9 +509,11 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     __syncwarp();
     tc::bar_or(kComputeBar, kCompute, false);
     float* red = reinterpret_cast<float*>(sm + kOffRed);  // [64][16]
-    if (loss_warp && lane < 16) {
-#pragma unroll
-      for (int o = 0; o < kNO; ++o) red[row * 16 + o] = dzsum[o];
+    if (loss_warp) {
+      red[row * 16 + c2] = dzsum[0];
+      red[row * 16 + c2 + 1] = dzsum[1];
+    }
+    if (loss_warp && c2 == 0) {
       red[row * 16 + 8] = st_loss;
       red[row * 16 + 9] = st_pg;
       red[row * 16 + 10] = st_v;
