@@ -43,20 +43,19 @@ constexpr int kComputeBar = 1;
 constexpr int kWarpCols = kH / (kComputeWarps / 4);  // features per compute warp
 
 // shared memory (bytes from the 1024-aligned base)
-constexpr uint32_t kOffX = 0;                                  // [64][208] bf16
-constexpr uint32_t kOffH1hi = kOffX + kRows * kKP * 2;         // [64][144]
+constexpr uint32_t kXBytes = kRows * kKP * 2;
+constexpr uint32_t kOffX = 0;                                  // [2][64][208] bf16
+constexpr uint32_t kOffH1hi = kOffX + 2 * kXBytes;             // [64][144]; later dL/da1
 constexpr uint32_t kOffH1lo = kOffH1hi + kRows * kH1P * 2;
-constexpr uint32_t kOffDA2hi = kOffH1lo + kRows * kH1P * 2;    // [64][128]
-constexpr uint32_t kOffDA2lo = kOffDA2hi + kRows * kH * 2;
-constexpr uint32_t kOffH2hi = kOffDA2lo + kRows * kH * 2;      // [64][128]; later dL/da1
+constexpr uint32_t kOffH2hi = kOffH1lo + kRows * kH1P * 2;     // [64][128]; later dL/da2
 constexpr uint32_t kOffH2lo = kOffH2hi + kRows * kH * 2;
 constexpr uint32_t kOffDZhi = kOffH2lo + kRows * kH * 2;       // [64][16]
 constexpr uint32_t kOffDZlo = kOffDZhi + kRows * 16 * 2;
 constexpr uint32_t kOffPK = kOffDZlo + kRows * 16 * 2;         // packed weights
 constexpr uint32_t kOffSC = kOffPK + kPpoPackedBytes;          // [2][5][64] per-sample scalars
 constexpr uint32_t kSmemUsed = kOffSC + 2 * 5 * kRows * 4;
-constexpr uint32_t kOffRed = kOffDA2hi;                        // [64][16] f32 end-of-kernel sums
-static_assert(kOffH1hi == 26624 && kOffPK == 133120, "layout");
+constexpr uint32_t kOffRed = kOffH2hi;                         // [64][16] f32 end-of-kernel sums
+static_assert(kOffPK % 128 == 0 && kSmemUsed <= 232448 - 1024, "layout");
 // tensor memory columns
 constexpr uint32_t kTmAcc = 0, kTmDW1 = 128, kTmDW2 = 336, kTmDW3 = 480;
 
@@ -113,15 +112,15 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
 
 __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradArgs a) {
   extern __shared__ __align__(16) uint8_t sm[];  // no-swizzle operands need 16 B
-  // operands ready (threads -> MMA warp): X, h1, h2, dz, da2, da1
-  __shared__ __align__(8) uint64_t opnd_bar[6];
-  // products done (commit -> threads): L1, L2, logits, dL/dh2, dL/dh1, dW1 (the tile's last)
-  __shared__ __align__(8) uint64_t acc_bar[6];
+  // operands ready (threads -> MMA warp): h1, h2, dz, da2, da1; X of even and of odd tiles
+  __shared__ __align__(8) uint64_t opnd_bar[7];
+  // products done (commit -> threads): L1, L2, logits, dL/dh2, dL/dh1, dW1, dW2, dW3
+  __shared__ __align__(8) uint64_t acc_bar[8];
   __shared__ __align__(8) uint64_t wload_bar, drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
-  enum { kX = 0, kH1 = 1, kH2 = 2, kDZ = 3, kDA2 = 4, kDA1 = 5 };
-  enum { kL1 = 0, kL2 = 1, kZ = 2, kDH2 = 3, kDH1 = 4, kDW1 = 5 };
+  enum { kH1 = 0, kH2 = 1, kDZ = 2, kDA2 = 3, kDA1 = 4, kX = 5 };
+  enum { kL1 = 0, kL2 = 1, kZ = 2, kDH2 = 3, kDH1 = 4, kDW1 = 5, kDW2 = 6, kDW3 = 7 };
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_tiles = (int)(a.B / kRows);
@@ -132,10 +131,10 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
   const uint8_t* pk = sm + kOffPK;
 
   if (tid == 0) {
-    for (int i = 0; i < 6; ++i) {
+    for (int i = 0; i < 8; ++i) tc::mbar_init(&acc_bar[i], 1);
+    for (int i = 0; i < 7; ++i) {
       // X: the loader warps; dz: the eight warps that compute the samples' losses
-      tc::mbar_init(&opnd_bar[i], i == kX ? kLoaders : (i == kDZ ? 256 : kCompute));
-      tc::mbar_init(&acc_bar[i], 1);
+      tc::mbar_init(&opnd_bar[i], i >= kX ? kLoaders : (i == kDZ ? 256 : kCompute));
     }
     tc::mbar_init(&wload_bar, 1);
     tc::mbar_init(&drain_bar, 1);
@@ -178,16 +177,15 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       const uint64_t dX = kmaj(kOffX, kKP), dW1 = kmaj(kOffPK + kPkW1, kKP);
       const uint64_t dH1[2] = {kmaj(kOffH1hi, kH1P), kmaj(kOffH1lo, kH1P)};
       const uint64_t dW2 = kmaj(kOffPK + kPkW2, kH), dW2t = mnmaj(kOffPK + kPkW2, kH);
-      const uint64_t dH2[2] = {kmaj(kOffH2hi, kH), kmaj(kOffH2lo, kH)};
+      const uint64_t dH2[2] = {kmaj(kOffH2hi, kH), kmaj(kOffH2lo, kH)};  // h2, later dL/da2
       const uint64_t dW3[2] = {kmaj(kOffPK + kPkW3hi, kH), kmaj(kOffPK + kPkW3lo, kH)};
       const uint64_t dW3t[2] = {mnmaj(kOffPK + kPkW3hi, kH), mnmaj(kOffPK + kPkW3lo, kH)};
       const uint64_t dDZ[2] = {kmaj(kOffDZhi, 16), kmaj(kOffDZlo, 16)};
-      const uint64_t dDA2[2] = {kmaj(kOffDA2hi, kH), kmaj(kOffDA2lo, kH)};
-      const uint64_t tDA2[2] = {mnmaj(kOffDA2hi, kH), mnmaj(kOffDA2lo, kH)};
-      const uint64_t tH2[2] = {mnmaj(kOffH2hi, kH), mnmaj(kOffH2lo, kH)};  // h2, later dL/da1
-      const uint64_t tH1[2] = {mnmaj(kOffH1hi, kH1P), mnmaj(kOffH1lo, kH1P)};
+      const uint64_t tH2[2] = {mnmaj(kOffH2hi, kH), mnmaj(kOffH2lo, kH)};
+      const uint64_t tH1[2] = {mnmaj(kOffH1hi, kH1P), mnmaj(kOffH1lo, kH1P)};  // h1, later dL/da1
       const uint64_t tDZ[2] = {mnmaj(kOffDZhi, 16), mnmaj(kOffDZlo, 16)};
       const uint64_t tX = mnmaj(kOffX, kKP);
+      constexpr uint64_t kXBuf = kXBytes >> 4;                    // the second X buffer
       constexpr uint64_t kS16 = 16;                               // 256 B: 16 features
       constexpr uint64_t kSampK = 2ull * (kH / 8) * 128 >> 4;     // 16 samples of a 128-wide buffer
       constexpr uint64_t kSampK1 = 2ull * (kH1P / 8) * 128 >> 4;  // ... of h1 (144 wide)
@@ -199,15 +197,19 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         return ok;
       };
       // the three products of a split pair: hi*hi, hi*lo, lo*hi (lo*lo is below 2^-16)
+      // L1 of tile it: acc = X W1^T (13 K-steps of 16 features)
+      auto layer1 = [&](int it) {
+        if (!wait_opnd(kX + (it & 1), (uint32_t)(it >> 1) & 1u)) return false;
+#pragma unroll
+        for (int ks = 0; ks < kKP / 16; ++ks)
+          tc::mma_ss(tmem + kTmAcc, dX + kXBuf * (it & 1) + kS16 * ks, dW1 + kS16 * ks, idL, ks > 0);
+        tc::commit(&acc_bar[kL1]);
+        return true;
+      };
+      layer1(0);
       for (int it = 0; ok && it < n_it; ++it) {
         const uint32_t par = (uint32_t)it & 1u;
         const uint32_t fresh = it == 0 ? 0u : 1u;  // the first tile starts the gradient sums
-        // L1: acc = X W1^T (13 K-steps of 16 features)
-        if (!wait_opnd(kX, par)) break;
-#pragma unroll
-        for (int ks = 0; ks < kKP / 16; ++ks)
-          tc::mma_ss(tmem + kTmAcc, dX + kS16 * ks, dW1 + kS16 * ks, idL, ks > 0);
-        tc::commit(&acc_bar[kL1]);
         // L2: acc = (h1_hi + h1_lo) W2^T
         if (!wait_opnd(kH1, par)) break;
 #pragma unroll
@@ -237,28 +239,30 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
           for (int ks = 0; ks < kRows / 16; ++ks)
             tc::mma_ss(tmem + kTmDW3, tH2[p == 2 ? 1 : 0] + kSampK * ks, tDZ[p == 1 ? 1 : 0] + kSampKZ * ks,
                        id3, (p | ks) != 0 ? 1u : fresh);
-        // dL/dh1 = da2 W2 into acc (its commit also covers dW3: h2's rows may be reused),
-        // then dW2 += da2^T [h1 | 1] under epilogue 3
+        tc::commit(&acc_bar[kDW3]);
+        // dL/dh1 = da2 W2 into acc, then dW2 += da2^T [h1 | 1] under epilogue 3
         if (!wait_opnd(kDA2, par)) break;
 #pragma unroll
         for (int part = 0; part < 2; ++part)
 #pragma unroll
           for (int ks = 0; ks < kH / 16; ++ks)
-            tc::mma_ss(tmem + kTmAcc, dDA2[part] + kS16 * ks, dW2t + kSampK * ks, idH, (part | ks) != 0);
+            tc::mma_ss(tmem + kTmAcc, dH2[part] + kS16 * ks, dW2t + kSampK * ks, idH, (part | ks) != 0);
         tc::commit(&acc_bar[kDH1]);
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
           for (int ks = 0; ks < kRows / 16; ++ks)
-            tc::mma_ss(tmem + kTmDW2, tDA2[p == 2 ? 1 : 0] + kSampK * ks, tH1[p == 1 ? 1 : 0] + kSampK1 * ks,
+            tc::mma_ss(tmem + kTmDW2, tH2[p == 2 ? 1 : 0] + kSampK * ks, tH1[p == 1 ? 1 : 0] + kSampK1 * ks,
                        id2, (p | ks) != 0 ? 1u : fresh);
-        // dW1 += da1^T [x | 1]
+        tc::commit(&acc_bar[kDW2]);
+        // the next tile's L1, then under it and the next epilogue 1 dW1 += da1^T [x | 1]
         if (!wait_opnd(kDA1, par)) break;
+        if (it + 1 < n_it && !layer1(it + 1)) break;
 #pragma unroll
         for (int p = 0; p < 2; ++p)
 #pragma unroll
           for (int ks = 0; ks < kRows / 16; ++ks)
-            tc::mma_ss(tmem + kTmDW1, tH2[p] + kSampK * ks, tX + kSampKX * ks, id1, (p | ks) != 0 ? 1u : fresh);
+            tc::mma_ss(tmem + kTmDW1, tH1[p] + kSampK1 * ks, tX + kXBuf * (it & 1) + kSampKX * ks, id1, (p | ks) != 0 ? 1u : fresh);
         tc::commit(&acc_bar[kDW1]);
       }
       if (!ok) abort_flag = 1;
@@ -269,11 +273,10 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     // the permutation and loads its scalars; the observation words go 8 rows x 4 consecutive
     // words to a load (a load then touches 8 lines; a row or half a row per lane touched 32,
     // and the L1's passes over them held up the epilogues' shared-memory accesses by 1-1.5 K
-    // cycles a tile).  Everything is loaded one tile ahead, into registers; once the previous
-    // tile's last MMA has completed the words are written out as the X operand (feature D is
+    // cycles a tile).  Everything is loaded one tile ahead, into registers; once dW1 of the
+    // tile before the previous one has completed (two X buffers) the words are written out as the X operand (feature D is
     // the constant 1 that carries db1 through dW1), 16 lanes to a core matrix, with the scalar
-    // rows, and the tile is released.  The next tile's loads are issued once epilogue 1 is
-    // over.
+    // rows, and the tile is released.
     if (n_it > 0) {
       const int D = a.D, nw = D / 4;
       const int row0 = (warp - kLoadWarp) * 16;
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       bool ok = true;
       load_tile(0);
       for (int it = 0; it < n_it; ++it) {
-        if (it > 0 && ok) ok = tc::mbar_wait(&acc_bar[kDW1], (uint32_t)(it - 1) & 1u);
+        if (it > 1 && ok) ok = tc::mbar_wait(&acc_bar[kDW1], (uint32_t)(it - 2) & 1u);
         ok = __all_sync(0xFFFFFFFFu, ok) && !abort_flag;
         if (!ok) break;
         float* scw = reinterpret_cast<float*>(sm + kOffSC) + (it & 1) * 5 * kRows;
@@ -314,14 +317,14 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         for (int t = 0; t < 2; ++t)
 #pragma unroll
           for (int k = 0; k < kQuads; ++k)
-            *reinterpret_cast<uint2*>(sm + kOffX + canon(row0 + 8 * t + rr, 16 * k + 4 * w0, kKP)) =
+            *reinterpret_cast<uint2*>(sm + kOffX + (it & 1) * kXBytes + canon(row0 + 8 * t + rr, 16 * k + 4 * w0, kKP)) =
                 make_uint2(tc::bytes_to_bf16x2(ow[t][k], 0), tc::bytes_to_bf16x2(ow[t][k], 2));
         if (lane < 16) {
 #pragma unroll
           for (int k = 0; k < 5; ++k) scw[k * kRows + row0 + lane] = sc[k];
         }
         tc::fence_proxy_async();
-        tc::mbar_arrive(&opnd_bar[kX]);
+        tc::mbar_arrive(&opnd_bar[kX + (it & 1)]);
         if (it + 1 < n_it) {
           load_tile(it + 1);
         }
@@ -366,7 +369,8 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       tc::wait_ld();
     };
     // tanh(acc + bias) -> hi | lo bf16 rows at dst (row width W)
-    auto act_rows = [&](const float* bias, uint32_t dst_hi, uint32_t dst_lo, int W) {
+    // once `free` says that nothing reads what was there before
+    auto act_rows = [&](const float* bias, uint32_t dst_hi, uint32_t dst_lo, int W, auto&& free) {
       const uint32_t dst = frag_addr(dst_hi, dst_lo, W) + (uint32_t)c0 * 16u;
       uint64_t bb[kWarpCols / 8];
 #pragma unroll
@@ -374,27 +378,28 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         bb[b] = *reinterpret_cast<const uint64_t*>(bias + c0 + 8 * b + c2);
       uint32_t v[kWarpCols / 8][4];
       acc_frags(v);
+      uint32_t o[kWarpCols / 8][4];
 #pragma unroll
-      for (int b = 0; b < kWarpCols / 8; ++b) {
-        uint32_t o[4];
+      for (int b = 0; b < kWarpCols / 8; ++b)
 #pragma unroll
         for (int h = 0; h < 2; ++h)
           tc::split_bf16x2_p(
               tc::tanh2(tc::f2_add(tc::f2_pack(__uint_as_float(v[b][2 * h]), __uint_as_float(v[b][2 * h + 1])), bb[b])),
-              o[h], o[2 + h]);
-        st_matrix_x4(dst + 128u * b, o);
-      }
+              o[b][h], o[b][2 + h]);
+      free();
+#pragma unroll
+      for (int b = 0; b < kWarpCols / 8; ++b) st_matrix_x4(dst + 128u * b, o[b]);
     };
-    // g (1 - h^2), h = hi + lo from the rows at src (row width W), -> hi | lo rows at dst
-    auto grad_rows = [&](uint32_t src_hi, uint32_t src_lo, int W, uint32_t dst_hi, uint32_t dst_lo) {
-      const uint32_t src = frag_addr(src_hi, src_lo, W) + (uint32_t)c0 * 16u;
-      const uint32_t dst = frag_addr(dst_hi, dst_lo, kH) + (uint32_t)c0 * 16u;
+    // g (1 - h^2), h = hi + lo from the rows at hi, lo (row width W), over those rows, likewise
+    auto grad_rows = [&](uint32_t hi, uint32_t lo, int W, auto&& free) {
+      const uint32_t at = frag_addr(hi, lo, W) + (uint32_t)c0 * 16u;
       uint32_t v[kWarpCols / 8][4];
       acc_frags(v);
+      uint32_t o[kWarpCols / 8][4];
 #pragma unroll
       for (int b = 0; b < kWarpCols / 8; ++b) {
-        uint32_t hv[4], o[4];
-        ld_matrix_x4(src + 128u * b, hv);
+        uint32_t hv[4];
+        ld_matrix_x4(at + 128u * b, hv);
 #pragma unroll
         for (int h2 = 0; h2 < 2; ++h2) {
           float h0a, h0b, h1a, h1b;
@@ -403,28 +408,32 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
           const uint64_t h = tc::f2_add(tc::f2_pack(h0a, h1a), tc::f2_pack(h0b, h1b));
           const uint64_t one_m = tc::f2_fma(h, tc::f2_sub(0ull, h), tc::f2_pack(1.0f, 1.0f));  // 1 - h^2
           const uint64_t g = tc::f2_pack(__uint_as_float(v[b][2 * h2]), __uint_as_float(v[b][2 * h2 + 1]));
-          tc::split_bf16x2_p(tc::f2_mul(g, one_m), o[h2], o[2 + h2]);
+          tc::split_bf16x2_p(tc::f2_mul(g, one_m), o[b][h2], o[b][2 + h2]);
         }
-        st_matrix_x4(dst + 128u * b, o);
       }
+      free();
+#pragma unroll
+      for (int b = 0; b < kWarpCols / 8; ++b) st_matrix_x4(at + 128u * b, o[b]);
     };
     // A wait that ran out ends this warp's loop; the others' waits then run out as well (each
     // is bounded) and all meet again below.
 
     for (int it = 0; it < n_it; ++it) {
       const uint32_t par = (uint32_t)it & 1u;
-      // the loader wrote this tile's X and scalars, after the previous tile's last MMA:
-      // every operand buffer is free again
-      if (!bad && !tc::mbar_wait(&opnd_bar[kX], par)) bad = true;
+      // the loader wrote this tile's scalars
+      if (!bad && !tc::mbar_wait(&opnd_bar[kX + (it & 1)], (uint32_t)(it >> 1) & 1u)) bad = true;
       // ---- epilogue 1: h1 = tanh(acc + b1) -> hi | lo rows -------------------------
       wait_acc(kL1, par);
       if (bad) break;
-      act_rows(b1, kOffH1hi, kOffH1lo, kH1P);
+      act_rows(b1, kOffH1hi, kOffH1lo, kH1P, [&] {  // the previous tile's dL/da1 is there
+        if (it > 0) wait_acc(kDW1, par ^ 1u);
+      });
+      if (bad) break;
       release(kH1);
       // ---- epilogue 2: h2 = tanh(acc + b2) -> hi | lo rows -------------------------
       wait_acc(kL2, par);
       if (bad) break;
-      act_rows(b2, kOffH2hi, kOffH2lo, kH);
+      act_rows(b2, kOffH2hi, kOffH2lo, kH, [] {});  // L2 came after the previous dW2
       release(kH2);
       // ---- the samples' losses and dL/dz: four lanes to a sample, two outputs each (the
       // fragment of the 8 output columns); the first group's warps take the quadrant's samples
@@ -495,12 +504,14 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
       // ---- dL/da2 = (dz W3) (1 - h2^2) --------------------------------------------
       wait_acc(kDH2, par);
       if (bad) break;
-      grad_rows(kOffH2hi, kOffH2lo, kH, kOffDA2hi, kOffDA2lo);
+      grad_rows(kOffH2hi, kOffH2lo, kH, [&] { wait_acc(kDW3, par); });
+      if (bad) break;
       release(kDA2);
-      // ---- epilogue 3: dL/da1 = (da2 W2) (1 - h1^2) into the h2 rows ----------------
+      // ---- epilogue 3: dL/da1 = (da2 W2) (1 - h1^2) over the h1 rows -----------------
       wait_acc(kDH1, par);
       if (bad) break;
-      grad_rows(kOffH1hi, kOffH1lo, kH1P, kOffH2hi, kOffH2lo);
+      grad_rows(kOffH1hi, kOffH1lo, kH1P, [&] { wait_acc(kDW2, par); });
+      if (bad) break;
       release(kDA1);
     }
     if (n_it > 0 && !bad) wait_acc(kDW1, (uint32_t)(n_it - 1) & 1u);  // the last dW1 (all MMAs)
