@@ -450,7 +450,17 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         tc::wait_ld();
         const float z[2] = {__uint_as_float(warp < 4 ? zr[0] : zr[2]) + b3[c2],
                             __uint_as_float(warp < 4 ? zr[1] : zr[3]) + b3[c2 + 1]};
-        auto sum4 = [&](float x) {  // over a sample's four lanes
+        // one after the other over a sample's four lanes: a sum over the outputs in their order
+        auto chain = [&](auto&& add) {
+          float x = add(0.f);
+#pragma unroll
+          for (int k = 1; k < 4; ++k) {
+            const float before = __shfl_up_sync(0xFFFFFFFFu, x, 1, 4);
+            if ((lane & 3) == k) x = add(before);
+          }
+          return __shfl_sync(0xFFFFFFFFu, x, 3, 4);
+        };
+        auto pick4 = [&](float x) {  // the one lane's value (the others hold 0)
           x += __shfl_xor_sync(0xFFFFFFFFu, x, 1);
           return x + __shfl_xor_sync(0xFFFFFFFFu, x, 2);
         };
@@ -458,19 +468,23 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
         float mx = fmaxf(c2 < A ? z[0] : -FLT_MAX, c2 + 1 < A ? z[1] : -FLT_MAX);
         mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
-        const float se = sum4((c2 < A ? __expf(z[0] - mx) : 0.f) + (c2 + 1 < A ? __expf(z[1] - mx) : 0.f));
+        const float e0 = c2 < A ? __expf(z[0] - mx) : 0.f, e1 = c2 + 1 < A ? __expf(z[1] - mx) : 0.f;
+        const float se = chain([&](float x) { return (x + e0) + e1; });
         const float lse = mx + __logf(se);
-        float logp[2], prob[2], ent_l = 0.f, lp_l = 0.f, v_l = 0.f;
+        float logp[2], prob[2], lp_l = 0.f, v_l = 0.f;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           const int o = c2 + k;
           logp[k] = z[k] - lse;
           prob[k] = o < A ? __expf(logp[k]) : 0.f;
-          if (o < A) ent_l -= prob[k] * logp[k];
           if (o == act) lp_l = logp[k];
           if (o == A) v_l = z[k];
         }
-        const float lp_a = sum4(lp_l), V = sum4(v_l), ent = sum4(ent_l);
+        const float lp_a = pick4(lp_l), V = pick4(v_l);
+        const float ent = chain([&](float x) {
+          x = c2 < A ? fmaf(-prob[0], logp[0], x) : x;
+          return c2 + 1 < A ? fmaf(-prob[1], logp[1], x) : x;
+        });
         const float rho = __expf(lp_a - lp_old);
         const float rho_c = fminf(fmaxf(rho, 1.0f - eps), 1.0f + eps);
         const float un = rho * adv_n, cl = rho_c * adv_n;
