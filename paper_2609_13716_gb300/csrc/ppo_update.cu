@@ -7,7 +7,8 @@
 // minibatch.  Per tile the forward (L1, L2 and the output layer as tcgen05 MMAs), the
 // per-sample loss gradient, and the backward run in one pass; the weight gradients
 // accumulate in tensor memory over the CTA's tiles (dW1 208 columns, dW2 144, dW3^T 16,
-// the working accumulator 128: 496 of 512) and leave once, as the CTA's partial sum.  Operands live in shared memory as rows of samples (8 x 16-byte core matrices, 8
+// the working accumulator 128: 496 of 512) and leave once, as the CTA's partial sum.
+// Operands live in shared memory as rows of samples (8 x 16-byte core matrices, 8
 // samples x 8 features): the same buffer is the K-major A operand of a forward product
 // (samples as M) and the MN-major operand of a weight-gradient product (samples as K).
 // Forward and backward products run with M = 64, whose 64 rows are the first 16
@@ -26,13 +27,13 @@ constexpr int kRows = kPpoTile;      // samples per tile
 constexpr int kKP = kPpoKP;          // padded input width: obs + the bias column + zeros
 constexpr int kH = kPpoHidden;       // hidden width
 constexpr int kH1P = 144;            // h1 row width as the B operand of dW2 (+ ones + pad)
-constexpr int kNO = 8;               // output rows (actions + value), padded
 // A tile is a chain of five products with an epilogue after each, so what bounds the kernel
 // is the epilogues' issue rate and the hand-over between them.  Sixteen compute warps, four
 // per scheduler: warp w takes the 16 samples of quadrant w % 4 and the 32 features of group
 // w / 4, as the 8 x 8 fragments that 16-lane tensor-memory loads, ldmatrix and stmatrix
 // share.  (With M = 128 over the tile's 64 rows only the warps of two schedulers could reach
-// the results: 10.3 against 8.4 ms for 4 epochs x 4 minibatches of 2 M samples.)
+// the results: 10.3 against 8.4 ms for 4 epochs x 4 minibatches of 2 M samples; 6.8 ms with
+// the loader, the loss, the second X buffer and the partials' layout below.)
 constexpr int kComputeWarps = 16;
 constexpr int kCompute = 32 * kComputeWarps;
 constexpr int kMmaWarp = kComputeWarps;          // issues the MMAs
@@ -548,47 +549,29 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     }
   }
 
-  // ---- the CTA's partial gradient: tensor-memory rows out, in parameter order ---------
+  // ---- the CTA's partial gradient, columns of 128 units (W1 and W2 transposed, so that a
+  // warp's lanes, the units, store side by side; the reduction puts them in parameter order) --
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   float* part = a.partials + (int64_t)blockIdx.x * a.part_stride;
-  if (!abort_flag && warp < 4) {
-    const int o = warp * 32 + lane;  // tensor-memory lane = output unit (dW1, dW2) / input (dW3^T)
-    const uint32_t lb = (uint32_t)(warp * 32) << 16;
-    const int D = a.D, A1 = a.n_act + 1;
-    for (int c0 = 0; c0 < kKP; c0 += 16) {
-      uint32_t v[16];
-      tc::ld_x16(tmem + kTmDW1 + lb + c0, v);
-      tc::wait_ld();
+  if (!abort_flag && warp < kComputeWarps) {
+    const int o = (warp & 3) * 32 + lane;  // tensor-memory lane = output unit (dW1, dW2) / input (dW3^T)
+    const uint32_t lb = (uint32_t)((warp & 3) * 32) << 16;
+    // columns [0, n) of the accumulator at tm -> rows of 128 at out, 16 columns a warp
+    auto dump = [&](uint32_t tm, int n, float* out) {
+      for (int c0 = 16 * (warp >> 2); c0 < n; c0 += 16 * (kComputeWarps / 4)) {
+        uint32_t v[16];
+        tc::ld_x16(tmem + tm + lb + c0, v);
+        tc::wait_ld();
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int c = c0 + k;
-        if (n_it == 0) v[k] = 0u;
-        if (c < D) part[a.oW1 + (int64_t)o * D + c] = __uint_as_float(v[k]);
-        else if (c == D) part[a.ob1 + o] = __uint_as_float(v[k]);
+        for (int k = 0; k < 16; ++k)
+          if (c0 + k < n) out[(int64_t)(c0 + k) * kH + o] = n_it == 0 ? 0.f : __uint_as_float(v[k]);
       }
-    }
-    for (int c0 = 0; c0 < kH1P; c0 += 16) {
-      uint32_t v[16];
-      tc::ld_x16(tmem + kTmDW2 + lb + c0, v);
-      tc::wait_ld();
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int c = c0 + k;
-        if (n_it == 0) v[k] = 0u;
-        if (c < kH) part[a.oW2 + (int64_t)o * kH + c] = __uint_as_float(v[k]);
-        else if (c == kH) part[a.ob2 + o] = __uint_as_float(v[k]);
-      }
-    }
-    {
-      uint32_t v[16];
-      tc::ld_x16(tmem + kTmDW3 + lb, v);
-      tc::wait_ld();
-#pragma unroll
-      for (int jj = 0; jj < kNO; ++jj)
-        if (jj < A1) part[a.oW3 + (int64_t)jj * kH + o] = n_it == 0 ? 0.f : __uint_as_float(v[jj]);
-    }
+    };
+    dump(kTmDW1, a.D + 1, part + a.oW1);  // W1, then b1
+    dump(kTmDW2, kH + 1, part + a.oW2);   // W2, then b2
+    dump(kTmDW3, a.n_act + 1, part + a.oW3);
   }
   if (!abort_flag && tid < 16) {
     const float* red = reinterpret_cast<const float*>(sm + kOffRed);
@@ -674,36 +657,40 @@ cudaError_t launch_ppo_advstat(const float* adv, uint32_t S, int w, Key key, uin
 }
 
 // ---- sum of the CTAs' partial gradients (fp64, CTA order) and its squared norm --------
-__global__ void ppo_reduce_kernel(const float* __restrict__ partials, int G, int64_t stride,
-                                  int64_t n_params, double* grad, double* blocksq, float* stats,
-                                  float inv_b) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void ppo_reduce_kernel(const PpoLayout L, const float* __restrict__ partials, int G, int64_t stride,
+                                  double* grad, double* blocksq, float* stats, float inv_b) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double g = 0.0;
-  if (i < n_params) {
+  if (p < L.n_params) {
     // four interleaved fp32 chains (CTA c into chain c % 4), joined in fp64: a fixed order
     // that keeps the dependent-add chain a quarter as long (fp64 adds are slow here)
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     int c = 0;
     for (; c + 4 <= G; c += 4) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) acc[k] += partials[(int64_t)(c + k) * stride + i];
+      for (int k = 0; k < 4; ++k) acc[k] += partials[(int64_t)(c + k) * stride + p];
     }
-    for (int k = 0; c < G; ++c, ++k) acc[k] += partials[(int64_t)c * stride + i];
+    for (int k = 0; c < G; ++c, ++k) acc[k] += partials[(int64_t)c * stride + p];
     g = ((double)acc[0] + (double)acc[1]) + ((double)acc[2] + (double)acc[3]);
+    int64_t i = p;  // W1 and W2 lie transposed in the partials
+    if (p < L.ob1) i = (p % kH) * L.D + p / kH;
+    else if (p >= L.oW2 && p < L.ob2) i = L.oW2 + ((p - L.oW2) % kH) * kH + (p - L.oW2) / kH;
     grad[i] = g;
   }
   __shared__ double sq[256];
-  sq[threadIdx.x] = i < n_params ? g * g : 0.0;
+  sq[threadIdx.x] = g * g;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if ((int)threadIdx.x < o) sq[threadIdx.x] += sq[threadIdx.x + o];
     __syncthreads();
   }
   if (threadIdx.x == 0) blocksq[blockIdx.x] = sq[0];
-  if (blockIdx.x == 0 && threadIdx.x < 6 && stats) {
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && k < 6 && stats) {  // a warp per diagnostic (a serial sum waits on every load)
     double s = 0.0;
-    for (int c = 0; c < G; ++c) s += (double)partials[c * stride + n_params + threadIdx.x];
-    stats[threadIdx.x] = (float)(s * inv_b);
+    for (int c = lane; c < G; c += 32) s += (double)partials[c * stride + L.n_params + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
+    if (lane == 0) stats[k] = (float)(s * inv_b);
   }
 }
 
@@ -745,10 +732,17 @@ cudaError_t launch_ppo_pack(const PpoLayout& L, const float* params, uint8_t* pk
 // ---- global-norm clipping and Adam, then repack ---------------------------------------
 __global__ void ppo_adam_kernel(const PpoAdamArgs a) {
   __shared__ float scale;
+  __shared__ double sq[256];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < a.n_blocks; b += blockDim.x) s += a.blocksq[b];
+  sq[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {  // a fixed order, the same in every block
+    if ((int)threadIdx.x < o) sq[threadIdx.x] += sq[threadIdx.x + o];
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int b = 0; b < a.n_blocks; ++b) s += a.blocksq[b];
-    const double norm = sqrt(s);
+    const double norm = sqrt(sq[0]);
     scale = (a.max_grad_norm > 0.f && norm >= (double)a.max_grad_norm) ? (float)((double)a.max_grad_norm / norm) : 1.0f;
   }
   __syncthreads();
@@ -767,7 +761,7 @@ __global__ void ppo_adam_kernel(const PpoAdamArgs a) {
 cudaError_t launch_ppo_reduce_adam(const float* partials, int G, int64_t stride, const PpoAdamArgs& a,
                                    float* stats, float inv_b, bool step, cudaStream_t s) {
   const unsigned nb = (unsigned)((a.L.n_params + 255) / 256);
-  ppo_reduce_kernel<<<nb, 256, 0, s>>>(partials, G, stride, a.L.n_params, a.grad, a.blocksq, stats, inv_b);
+  ppo_reduce_kernel<<<nb, 256, 0, s>>>(a.L, partials, G, stride, a.grad, a.blocksq, stats, inv_b);
   if (step) ppo_adam_kernel<<<nb, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
