@@ -32,7 +32,7 @@ constexpr int kH1P = 144;            // h1 row width as the B operand of dW2 (+ 
 // per scheduler: warp w takes the 16 samples of quadrant w % 4 and the 32 features of group
 // w / 4, as the 8 x 8 fragments that 16-lane tensor-memory loads, ldmatrix and stmatrix
 // share.  (With M = 128 over the tile's 64 rows only the warps of two schedulers could reach
-// the results: 10.3 against 8.4 ms for 4 epochs x 4 minibatches of 2 M samples; 6.8 ms with
+// the results: 10.3 against 8.4 ms for 4 epochs x 4 minibatches of 2 M samples; 6.7 ms with
 // the loader, the loss, the second X buffer and the partials' layout below.)
 constexpr int kComputeWarps = 16;
 constexpr int kCompute = 32 * kComputeWarps;
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
 #pragma unroll
           for (int k = 1; k < 4; ++k) {
             const float before = __shfl_up_sync(0xFFFFFFFFu, x, 1, 4);
-            if ((lane & 3) == k) x = add(before);
+            x = add((lane & 3) == 0 ? 0.f : before);
           }
           return __shfl_sync(0xFFFFFFFFu, x, 3, 4);
         };
@@ -562,6 +562,7 @@ __global__ void __launch_bounds__(kThreadsPpo, 1) ppo_grad_kernel(const PpoGradA
     const uint32_t lb = (uint32_t)((warp & 3) * 32) << 16;
     // columns [0, n) of the accumulator at tm -> rows of 128 at out, 16 columns a warp
     auto dump = [&](uint32_t tm, int n, float* out) {
+#pragma unroll 1
       for (int c0 = 16 * (warp >> 2); c0 < n; c0 += 16 * (kComputeWarps / 4)) {
         uint32_t v[16];
         tc::ld_x16(tmem + tm + lb + c0, v);
